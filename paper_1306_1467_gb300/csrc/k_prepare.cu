@@ -399,64 +399,109 @@ static cudaError_t launch_sort_ipt(const int32_t *ii_t, int ii_stride, int w, co
 
 // ---- K3, packed variant (the one every row goes through first) ---------------------------
 // The same stable sort for rows whose items fit one 32-bit word: value - min
-// in the high bits above a sample index of ib bits (ib = 14 up to 16,384
-// samples with 512-thread CTAs, two per SM; 15 above, with 1024-thread CTAs).
+// in the high bits above a sample index of ib bits (14 up to 16,384 samples).
 // A row whose value span does not fit next to its index is listed for the
-// two-word sort above.  Only the value bits are sorted, in one pass when the
-// span has at most 9 bits and in two passes over digits of half the span's
-// bits (5 to 9) otherwise; the starting index order and stable passes order
-// ties by sample index.  A pass ranks each item once: while the warps count
-// their digits (the lanes holding the same digit come from one ballot per
-// digit bit), every item records its rank among its warp's earlier items of
-// the same digit (in shared memory, or two 16-bit ranks per register), so the
-// scatter after the CTA-wide scan needs only the scanned offsets.  Then the
-// bank choice of the two weight copies and the run-interleaved write, one
-// 16-byte chunk per thread.
-constexpr int kPkThreads = 512;
-constexpr int kPkRefinePasses = 1;  // a second pass buys no search time
-constexpr int kPkDigitBits = 9;
+// two-word sort above.  Only the value bits are sorted, in passes over digits
+// of at most 8 bits, as few and as even as that allows (at least 5 bits: one
+// pass up to 8 bits of span, two up to 16); the starting index order and stable
+// passes order ties by sample index.
+//
+// A pass: each warp counts the digits of its items (a contiguous range of
+// positions) in counters of its own, the counters become first positions by a
+// scan over (digit, warp), and each item takes its place with an atomic add on
+// its warp's counter of its digit, 32 items after the 32 before them.  That is
+// stable where the lanes of one such add are served in lane order, as this GPU
+// does; since nothing promises it, the write checks that the finished row's
+// words ascend (a word is value, then sample index, so ascending words are the
+// order itself) and a row that fails is listed for the two-word sort, which
+// ranks with ballots.
+//
+// Then the bank choice of the two weight copies and the run-interleaved write,
+// one 16-byte chunk per thread.
+//
+// What bounds it: shared memory.  16x16 / 15,000 (ncu): shared-memory pipe 66%
+// busy (37 wavefronts per 32 items, half of them the atomics' bank conflicts),
+// issue 49%, ALU 53%, 132 instructions an item.  Ranking with one ballot per
+// digit bit, the form before, was ALU bound at 223 instructions an item.
+// Tables in all, before -> now: 24x24 / 2,003 6.04 -> 2.90 ms, 32x32 / 5,003
+// 31.9 -> 20.0, 24x24 / 15,000 20.9 -> 16.1, 24x24 / 18,300 34.4 -> 26.0.
+//
+// Threads per CTA grow with the row (128 up to 4,096 samples, 256 up to 8,192,
+// 512 up to 16,384), 1,024 threads an SM in all: small CTAs leave other rows
+// to run while one waits at a barrier (24x24 / 2,003 in 512-thread CTAs: twice
+// the time).  From 16,385 to 20,480 samples two CTAs of 640 threads still fit
+// an SM (18,300: 26.0 ms, 29.9 with one CTA of 1,024); above, one of 1,024.
+//
+// Measured and dropped: one pass with a counter per value for spans up to 14
+// bits (one warp ranking a row in order waits its turn behind the other CTA's
+// warps: 16.9 ms at 15,000); buckets filled in any order and put right by
+// counting or by insertion (28.7 ms); predicated atomics for the last warp's
+// missing items (the compiler wraps each in a branch: 158 instructions).
+constexpr int kPkDigitBits = 8;
 constexpr int kPkRadix = 1 << kPkDigitBits;
 
-__host__ __device__ constexpr bool packed_ranks_in_smem(int ipt, int th) { return th <= 512 && ipt >= 20 && ipt <= 30; }
+// Adds to counters in shared memory, as the instructions themselves: the
+// ranking depends on one following the other in program order.
+__device__ __forceinline__ void shared_add(uint32_t addr, uint32_t x) {
+    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
+}
+__device__ __forceinline__ uint32_t shared_take(uint32_t addr) {
+    uint32_t old;
+    asm volatile("atom.shared.add.u32 %0, [%1], 1;" : "=r"(old) : "r"(addr) : "memory");
+    return old;
+}
 
 template <int IPT, int TH>
-__global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1)
+__global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
     k_sort_rows_packed(const int32_t *__restrict__ ii_t, const uint16_t *__restrict__ ii16, int ii_stride, int w,
                        const DevFeature *__restrict__ feat, int64_t f0, WeightLayout L,
                        uint16_t *__restrict__ rows, int npad, int32_t *ovf, int32_t *stat) {
     constexpr int NP = TH * IPT;
-    constexpr int WARPS = TH / 32, HSTRIDE = WARPS + 1, HWORDS = kPkRadix * HSTRIDE;
+    constexpr int WARPS = TH / 32;
     constexpr int GROUPS = NP / 32;  // lane-run groups of the longest row
-    static_assert(3 * GROUPS * 4 <= HWORDS * (packed_ranks_in_smem(IPT, TH) ? 2 : 4),
-                  "histogram space too small for the refine list");
-    // 512-thread CTAs of 20 to 30 items keep the items' ranks in shared memory
-    // (registers would spill) and count in 16 bits (counts and offsets stay
-    // below 2^16) so that two CTAs still fit an SM; the others keep them in
-    // registers
-    constexpr bool RS = packed_ranks_in_smem(IPT, TH);
-    using HT = typename std::conditional<RS, uint16_t, uint32_t>::type;
+    static_assert(4 * GROUPS <= kPkRadix * WARPS, "counter space too small for the refine list");
     const int n = L.n;
     extern __shared__ __align__(16) uint8_t smem[];
     uint32_t *skey = reinterpret_cast<uint32_t *>(smem);                        // NP items
-    uint16_t *rks = reinterpret_cast<uint16_t *>(skey + NP);                   // NP ranks (RS)
-    HT *hist = reinterpret_cast<HT *>(RS ? (uint8_t *)(rks + NP) : (uint8_t *)(skey + NP));  // HWORDS
-    uint32_t *gchoice = reinterpret_cast<uint32_t *>(
-        reinterpret_cast<uint8_t *>(hist) + (((size_t)HWORDS * sizeof(HT) + 15) & ~(size_t)15));  // GROUPS
-    uint32_t *ws = gchoice + GROUPS;                                            // WARPS
-    int32_t *mm = reinterpret_cast<int32_t *>(ws + WARPS);                      // 2
+    // kPkRadix * WARPS counters, from a multiple of a warp's share of them
+    uint32_t *hist = skey + NP + ((0u - smem_u32(skey + NP)) & (4u * kPkRadix - 1u)) / 4u;
+    uint32_t *gchoice = hist + kPkRadix * WARPS;                                // GROUPS
+    uint32_t *ws = gchoice + GROUPS;                                            // kPkRadix / 32
+    int32_t *mm = reinterpret_cast<int32_t *>(ws + kPkRadix / 32);              // 2 * WARPS
+    uint32_t *spare = reinterpret_cast<uint32_t *>(mm + 2 * WARPS);             // 32
 
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int pos0 = wp * 32 * IPT + lane;
     const DevFeature d = feat[f0 + blockIdx.x];
 
     // the feature on every window (K2's arithmetic), four windows per thread
-    // and corner load; boxes of at most kNarrowArea pixels from the integral
-    // images modulo 2^16 (half the bytes)
+    // and corner load.  Boxes of at most kNarrowArea pixels come from the
+    // integral images modulo 2^16, two windows to a 32-bit word (half the
+    // bytes, and the corners are added two windows at a time); they are kept
+    // as 16-bit offsets from the type's smallest possible value.
+    const bool narrow = ii16 && d.w * d.h <= kNarrowArea;
+    uint16_t *val16 = reinterpret_cast<uint16_t *>(skey);
     int32_t lo = INT_MAX, hi = INT_MIN;
-    auto values = [&](auto value4) {
+    if (narrow) {
+        uint32_t lo2 = 0xffffffffu, hi2 = 0u;
         for (int q = threadIdx.x; 4 * q < n; q += TH) {
             const int p = 4 * q;
-            const int4 x = value4(p);
+            uint2 x = haar_offsets4(ii16, ii_stride, w, d.type, d.x, d.y, d.w, d.h, p);
+            if (p + 4 > n) {  // past the last sample: repeat the last one's
+                if (p + 1 >= n) x.x = (x.x & 0xffffu) * 0x10001u;
+                if (p + 2 >= n) x.y = (x.x >> 16) * 0x10001u;
+                else x.y = (x.y & 0xffffu) * 0x10001u;
+            }
+            reinterpret_cast<uint2 *>(skey)[q] = x;
+            lo2 = __vminu2(lo2, __vminu2(x.x, x.y));
+            hi2 = __vmaxu2(hi2, __vmaxu2(x.x, x.y));
+        }
+        lo = (int32_t)min(lo2 & 0xffffu, lo2 >> 16);
+        hi = (int32_t)max(hi2 & 0xffffu, hi2 >> 16);
+    } else {
+        for (int q = threadIdx.x; 4 * q < n; q += TH) {
+            const int p = 4 * q;
+            const int4 x = haar_value4(ii_t, ii_stride, w, d.type, d.x, d.y, d.w, d.h, p);
             reinterpret_cast<uint4 *>(skey)[q] = make_uint4((uint32_t)x.x, (uint32_t)x.y, (uint32_t)x.z, (uint32_t)x.w);
             lo = min(lo, x.x);
             hi = max(hi, x.x);
@@ -464,216 +509,218 @@ __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1)
             if (p + 2 < n) { lo = min(lo, x.z); hi = max(hi, x.z); }
             if (p + 3 < n) { lo = min(lo, x.w); hi = max(hi, x.w); }
         }
-    };
-    if (ii16 && d.w * d.h <= kNarrowArea)
-        values([&](int p) { return haar_value4_narrow(ii16, ii_stride, w, d.type, d.x, d.y, d.w, d.h, p); });
-    else
-        values([&](int p) { return haar_value4(ii_t, ii_stride, w, d.type, d.x, d.y, d.w, d.h, p); });
-#pragma unroll
-    for (int s = 16; s; s >>= 1) {
-        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, s));
-        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, s));
     }
-    if (threadIdx.x == 0) { mm[0] = INT_MAX; mm[1] = INT_MIN; }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) { mm[2 * wp] = lo; mm[2 * wp + 1] = hi; }
     __syncthreads();
-    if (lane == 0) { atomicMin(&mm[0], lo); atomicMax(&mm[1], hi); }
-    __syncthreads();
-    lo = mm[0];
-    hi = mm[1];
+    lo = __reduce_min_sync(0xffffffffu, mm[2 * (lane % WARPS)]);
+    hi = __reduce_max_sync(0xffffffffu, mm[2 * (lane % WARPS) + 1]);
     const uint32_t span = static_cast<uint32_t>(hi) - static_cast<uint32_t>(lo);
     const int bits = span ? 32 - __clz(span) : 0;
-    const int ib = 32 - __clz((uint32_t)(n - 1));  // bits of a sample index
+    // bits of a sample index (at least those the bank choice looks at)
+    const int ib = max(10, 32 - __clz((uint32_t)(n - 1)));
     const uint32_t imask = (1u << ib) - 1u;
     if (bits + ib > 32) {  // value and index do not fit one word: the two-word sort takes the row
         if (threadIdx.x == 0) ovf[1 + atomicAdd(ovf, 1)] = (int32_t)blockIdx.x;
         return;
     }
-    uint32_t c[IPT];
+    // items pos0 + 32 j; those from j = mine on lie past the last sample and
+    // are not counted or stored
+    const int mine = (n - pos0 + 31) >> 5;
+    // a warp with samples to the end of its range counts and places all of them;
+    // another's lanes past the last sample add to a spare word (a skipped add
+    // costs a branch around every one)
+    const bool all_mine = (wp + 1) * 32 * IPT <= n;
+    const uint32_t spare32 = smem_u32(spare + lane);
+    const int passes = max(1, (bits + kPkDigitBits - 1) / kPkDigitBits);
+    const int D = max(5, (bits + passes - 1) / passes);
+    uint32_t *own = hist + (wp << D);  // this warp's counters, one per digit
+    const uint32_t own32 = smem_u32(own);
+    const uint32_t dmask = ((1u << D) - 1u) << 2;  // a digit as a byte offset
+    // one stable pass over the D-bit digit from bit `shift` of the values, the
+    // items in position order from item(j, p)
+    auto radix_pass = [&](int shift, auto item) {
+        const int sh = ib + shift - 2;
+        for (int k = lane; k < (1 << D); k += 32) own[k] = 0u;
+        __syncwarp();
+        auto count = [&](auto whole) {
 #pragma unroll
-    for (int j = 0; j < IPT; ++j) {
-        const int p = pos0 + j * 32;
-        // padding items take the all-ones word: they sort after every real item
-        c[j] = (p < n) ? (((skey[p] - static_cast<uint32_t>(lo)) << ib) | (uint32_t)p) : 0xffffffffu;
-    }
-    __syncthreads();
-
-    const uint32_t lt = lanemask_lt();
-    // one stable pass over the D-bit digit at value bit `shift`; the sorted
-    // items end in skey and in c
-    auto radix_pass = [&](auto dbits, int shift) {
-        constexpr int D = decltype(dbits)::value;
-        constexpr uint32_t DMASK = (1u << D) - 1u;
-        // counts warp-major (warp w's digit d at w * R + d): the lanes of a
-        // warp touch neighbouring words, whatever their digits
-        constexpr int R = (1 << D) + (sizeof(HT) == 2 ? 2 : 1);
-        static_assert(WARPS * R <= HWORDS, "histogram space too small");
-        const int sh = ib + shift;
-        for (int k = threadIdx.x; k < WARPS * R; k += TH) hist[k] = 0;
+            for (int j = 0; j < IPT; ++j) {
+                const uint32_t at = ((item(j, pos0 + 32 * j) >> sh) & dmask) | own32;
+                shared_add(decltype(whole)::value || j < mine ? at : spare32, 1u);
+            }
+        };
+        if (all_mine) count(std::true_type{});
+        else count(std::false_type{});
         __syncthreads();
-        // each item's rank among the warp's earlier items of its digit, in
-        // position order (item j before item j + 1, lanes in order): in shared
-        // memory at the item's position (RS), else two per register
-        uint32_t rk[RS ? 1 : (IPT + 1) / 2];
+        // first positions, by digit, then warp: a thread takes digit q * TH +
+        // tid of every warp's counters
+        constexpr int ROUNDS = kPkRadix / TH > 0 ? kPkRadix / TH : 1;
+        uint32_t pre[ROUNDS];
 #pragma unroll
-        for (int j = 0; j < IPT; ++j) {
-            const uint32_t dg = (c[j] >> sh) & DMASK;
-            const uint32_t peers = digit_peers<D>(dg);
-            const int leader = __ffs(peers) - 1;
-            uint32_t old = 0;
-            if (lane == leader) {
-                old = hist[wp * R + dg];
-                hist[wp * R + dg] = (HT)(old + __popc(peers));
-            }
-            old = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & lt);
-            if constexpr (RS) {
-                rks[pos0 + j * 32] = (uint16_t)old;
-            } else {
-                if (j & 1) rk[j >> 1] |= old << 16;
-                else rk[j >> 1] = old;
-            }
-        }
-        __syncthreads();
-        {
-            constexpr int PER = (1 << D) * WARPS / TH;
-            static_assert(PER >= 1, "digit too narrow for the scan");
-            uint32_t cnt[PER];
-            uint32_t s = 0;
-#pragma unroll
-            for (int q = 0; q < PER; ++q) {
-                const int lin = threadIdx.x * PER + q;
-                cnt[q] = hist[(lin % WARPS) * R + lin / WARPS];
-                s += cnt[q];
-            }
-            // CTA-wide exclusive scan of the per-thread sums
-            uint32_t inc = s;
-#pragma unroll
-            for (int dd = 1; dd < 32; dd <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, inc, dd);
-                if (lane >= dd) inc += y;
-            }
-            if (lane == 31) ws[wp] = inc;
-            __syncthreads();
-            if (wp == 0) {
-                const uint32_t t = lane < WARPS ? ws[lane] : 0u;
-                uint32_t ti = t;
+        for (int q = 0; q < ROUNDS; ++q) {
+            const int dg = q * TH + (int)threadIdx.x;
+            if (dg < (1 << D)) {  // uniform over a warp: D >= 5
+                uint32_t t = 0u;
+#pragma unroll 8
+                for (int w = 0; w < WARPS; ++w) t += hist[(w << D) + dg];
+                uint32_t inc = t;
 #pragma unroll
                 for (int dd = 1; dd < 32; dd <<= 1) {
-                    const uint32_t y = __shfl_up_sync(0xffffffffu, ti, dd);
-                    if (lane >= dd) ti += y;
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, dd);
+                    if (lane >= dd) inc += y;
                 }
-                if (lane < WARPS) ws[lane] = ti - t;
-            }
-            __syncthreads();
-            uint32_t off = ws[wp] + inc - s;
-#pragma unroll
-            for (int q = 0; q < PER; ++q) {
-                const int lin = threadIdx.x * PER + q;
-                hist[(lin % WARPS) * R + lin / WARPS] = (HT)off;
-                off += cnt[q];
+                if (lane == 31) ws[q * WARPS + wp] = inc;
+                pre[q] = inc - t;
             }
         }
         __syncthreads();
 #pragma unroll
-        for (int j = 0; j < IPT; ++j) {
-            const uint32_t dg = (c[j] >> sh) & DMASK;
-            const uint32_t r = RS ? (uint32_t)rks[pos0 + j * 32] : ((rk[j >> 1] >> (16 * (j & 1))) & 0xffffu);
-            skey[hist[wp * R + dg] + r] = c[j];
+        for (int q = 0; q < ROUNDS; ++q) {
+            const int dg = q * TH + (int)threadIdx.x;
+            if (dg < (1 << D)) {
+                const int before = q * WARPS + wp;  // at most kPkRadix / 32 - 1
+                uint32_t run = pre[q] + __reduce_add_sync(0xffffffffu, lane < before ? ws[lane % (kPkRadix / 32)] : 0u);
+#pragma unroll 8
+                for (int w = 0; w < WARPS; ++w) {
+                    const uint32_t t = hist[(w << D) + dg];
+                    hist[(w << D) + dg] = run;
+                    run += t;
+                }
+            }
         }
-        __syncthreads();
-        // the next pass's first write to skey or hist follows two barriers
+        // the items again (holding them through the scan costs spills), all
+        // read before any is stored
+        uint32_t c[IPT];
 #pragma unroll
-        for (int j = 0; j < IPT; ++j) c[j] = skey[pos0 + j * 32];
+        for (int j = 0; j < IPT; ++j) c[j] = item(j, pos0 + 32 * j);
+        __syncthreads();
+        // (adds in batches, so that a store does not wait for its own add alone)
+        auto place = [&](auto whole) {
+            constexpr int BATCH = 4;
+#pragma unroll
+            for (int j0 = 0; j0 < IPT; j0 += BATCH) {
+                uint32_t to[BATCH];
+#pragma unroll
+                for (int u = 0; u < BATCH; ++u) {
+                    const int j = j0 + u;
+                    if (j >= IPT) break;
+                    const uint32_t at = ((c[j] >> sh) & dmask) | own32;
+                    to[u] = shared_take(decltype(whole)::value || j < mine ? at : spare32);
+                }
+#pragma unroll
+                for (int u = 0; u < BATCH; ++u) {
+                    const int j = j0 + u;
+                    if (j < IPT && (decltype(whole)::value || j < mine)) skey[to[u]] = c[j];
+                }
+            }
+        };
+        if (all_mine) place(std::true_type{});
+        else place(std::false_type{});
+        __syncthreads();
     };
-    // Two passes at most (value bits <= 18); the digit is as narrow as that
-    // allows (one ballot per digit bit), at least 5 bits.
-    if (bits > 0) {
-        const int passes = bits <= kPkDigitBits ? 1 : 2;
-        const int D = max(5, (bits + passes - 1) / passes);
-        for (int shift = 0; shift < bits; shift += D) {
-            switch (D) {
-                case 5: radix_pass(std::integral_constant<int, 5>{}, shift); break;
-                case 6: radix_pass(std::integral_constant<int, 6>{}, shift); break;
-                case 7: radix_pass(std::integral_constant<int, 7>{}, shift); break;
-                case 8: radix_pass(std::integral_constant<int, 8>{}, shift); break;
-                default: radix_pass(std::integral_constant<int, kPkDigitBits>{}, shift); break;
-            }
-        }
-    } else {
-        // one value: the items are already in order
-#pragma unroll
-        for (int j = 0; j < IPT; ++j) skey[pos0 + j * 32] = c[j];
-        __syncthreads();
-    }
+    // (a row of one value takes a pass too: every digit 0, the items in order)
+    if (narrow)
+        radix_pass(0, [&](int j, int p) { return (((uint32_t)val16[p] - (uint32_t)lo) << ib) + (uint32_t)p; });
+    else
+        radix_pass(0, [&](int j, int p) { return ((skey[p] - (uint32_t)lo) << ib) + (uint32_t)p; });
+    for (int shift = D; shift < bits; shift += D) radix_pass(shift, [&](int j, int p) { return skey[p]; });
 
     uint16_t *out = rows + (size_t)blockIdx.x * npad;
     const int run = npad / 32;
     if (L.dual) {
-        // bank-balanced copy choice per gather group (see k_sort_rows); the
-        // loads of the 32 banks as 2-bit counters in one 64-bit word (bank b
-        // at bits 2b, 2b + 1; a load above 3 counts as 3).  Only the groups
-        // left with a bank at 3 after the greedy pass get the pass of single
-        // moves; they are listed first (in the free histogram space) so that
-        // the threads share them evenly.
-        auto level = [](uint64_t C, int b) { return (uint32_t)(C >> (2 * b)) & 3u; };
-        auto inc = [&](uint64_t &C, int b) {
-            if (level(C, b) != 3u) C += 1ull << (2 * b);
+        // bank-balanced copy choice per gather group (see k_sort_rows): each
+        // entry goes to the less loaded of its two banks, one thread a group.
+        // The 32 banks' loads are three masks (banks with at least 1, 2, 3
+        // entries).  The groups left with a bank at 3 are listed (in the free
+        // counter space) and taken by a warp each, a lane per entry: while an
+        // entry of such a bank has its other bank below 2, the first of them
+        // moves there.
+        const bool part = L.nb < n;  // samples from nb on have one copy only
+        uint32_t *rlist = hist;      // (group, masks) of the groups to refine
+        auto bank_bits = [&](uint32_t x, uint32_t &a, uint32_t &b) {  // x: a word of skey (its bits 0-9 are the index's)
+            a = __funnelshift_l(0u, 1u, x);                    // 1 << (i mod 32)
+            b = __funnelshift_l(0u, 1u, x + 13u * (x >> 5));  // 1 << (rot_b(i) mod 32)
         };
-        auto dec = [&](uint64_t &C, int b) {
-            if (level(C, b) != 0u) C -= 1ull << (2 * b);
-        };
-        uint32_t *rlist = reinterpret_cast<uint32_t *>(hist);  // (group, counters lo, hi) of groups to refine
         if (threadIdx.x == 0) mm[0] = 0;
         __syncthreads();
         for (int g = threadIdx.x; g < run; g += TH) {
-            uint64_t C = 0;
-            uint32_t mask = 0;
+            uint32_t m1 = 0u, m2 = 0u, m3 = 0u, mask = 0u;
             const int kend = min(32, (n - g + run - 1) / run);  // entries k * run + g < n
-            for (int k = 0; k < kend; ++k) {
-                const int i = (int)(skey[k * run + g] & imask);
-                const int ba = i & 31, bb = rot_b(i) & 31;
-                const uint32_t la = level(C, ba), lb = level(C, bb);
-                const bool tob = i < L.nb && lb < la;
-                const int c = tob ? bb : ba;
-                if ((tob ? lb : la) != 3u) C += 1ull << (2 * c);
-                mask |= (uint32_t)tob << k;
+            auto entry = [&](int k) {
+                const uint32_t x = skey[k * run + g];
+                uint32_t a, b;
+                bank_bits(x, a, b);
+                if (part && (int)(x & imask) >= L.nb) b = a;
+                // bank b is less loaded if it has no entry and a has one, or
+                // has one and a has two; without branches
+                uint32_t to;
+                asm("{\n\t.reg .pred p, q;\n\t.reg .b32 t;\n\t"
+                    "and.b32 t, %2, %4;\n\tsetp.ne.u32 p, t, 0;\n\t"
+                    "and.b32 t, %2, %5;\n\tsetp.eq.and.u32 p, t, 0, p;\n\t"
+                    "and.b32 t, %3, %4;\n\tsetp.ne.u32 q, t, 0;\n\t"
+                    "and.b32 t, %3, %5;\n\tsetp.eq.and.u32 q, t, 0, q;\n\t"
+                    "or.pred p, p, q;\n\t"
+                    "selp.b32 %0, %5, %4, p;\n\t"
+                    "@p or.b32 %1, %1, %6;\n\t}"
+                    : "=r"(to), "+r"(mask)
+                    : "r"(m1), "r"(m2), "r"(a), "r"(b), "r"(1u << k));
+                m3 |= m2 & to;
+                m2 |= m1 & to;
+                m1 |= to;
+            };
+            if (kend == 32) {
+#pragma unroll 8
+                for (int k = 0; k < 32; ++k) entry(k);
+            } else {
+                for (int k = 0; k < kend; ++k) entry(k);
+                const uint32_t to = 1u << (n & 31);  // the padding word, read as a broadcast
+                m3 |= m2 & to;
+                m2 |= m1 & to;
+                m1 |= to;
             }
-            if (kend < 32) inc(C, n & 31);  // the padding word, read as a broadcast
             gchoice[g] = mask;
-            if (kPkRefinePasses > 0 && ((C & (C >> 1)) & 0x5555555555555555ull)) {
+            if (m3) {
                 const int q = atomicAdd(&mm[0], 1);
-                rlist[3 * q] = (uint32_t)g;
-                rlist[3 * q + 1] = (uint32_t)C;
-                rlist[3 * q + 2] = (uint32_t)(C >> 32);
+                rlist[4 * q] = (uint32_t)g;
+                rlist[4 * q + 1] = m1;
+                rlist[4 * q + 2] = m2;
+                rlist[4 * q + 3] = m3;
             }
         }
         __syncthreads();
         const int nref = mm[0];
-        for (int q = threadIdx.x; q < nref; q += TH) {
-            const int g = (int)rlist[3 * q];
-            uint64_t C = (uint64_t)rlist[3 * q + 1] | ((uint64_t)rlist[3 * q + 2] << 32);
+        for (int q = wp; q < nref; q += WARPS) {
+            const int g = (int)rlist[4 * q];
+            uint32_t m1 = rlist[4 * q + 1], m2 = rlist[4 * q + 2], m3 = rlist[4 * q + 3];
             uint32_t mask = gchoice[g];
-            const int kend = min(32, (n - g + run - 1) / run);
-            for (int pass = 0; pass < kPkRefinePasses; ++pass)
-                for (int k = 0; k < kend; ++k) {
-                    const int i = (int)(skey[k * run + g] & imask);
-                    if (i >= L.nb) continue;
-                    const int ba = i & 31, bb = rot_b(i) & 31;
-                    const bool onb = (mask >> k) & 1u;
-                    const int cur = onb ? bb : ba, oth = onb ? ba : bb;
-                    if (level(C, cur) > level(C, oth) + 1) {
-                        dec(C, cur);
-                        inc(C, oth);
-                        mask ^= 1u << k;
-                    }
-                }
-            gchoice[g] = mask;
+            const bool in = lane * run + g < n;
+            const uint32_t x = in ? skey[lane * run + g] : 0u;
+            uint32_t a, b;
+            bank_bits(x, a, b);
+            bool onb = (mask >> lane) & 1u;
+            const bool can = in && (int)(x & imask) < L.nb;
+            for (;;) {
+                const uint32_t cur = onb ? b : a, oth = onb ? a : b;
+                const uint32_t moves = __ballot_sync(0xffffffffu, can && (m3 & cur) && !(m2 & oth));
+                if (!moves) break;
+                const int first = __ffs(moves) - 1;
+                const uint32_t from = __shfl_sync(0xffffffffu, cur, first), to = __shfl_sync(0xffffffffu, oth, first);
+                m3 &= ~from;
+                m2 |= m1 & to;
+                m1 |= to;
+                mask ^= 1u << first;
+                if (lane == first) onb = !onb;
+            }
+            if (lane == 0) gchoice[g] = mask;
         }
         __syncthreads();
     }
     // the run-interleaved write: one 16-byte chunk (8 entries) per thread;
     // chunk c holds entries t * 8 .. t * 8 + 7 of lane run k (c = t * 32 + k),
     // consecutive positions p0 .. p0 + 7 of the value order
-    bool bad = false;
+    bool bad = false, unsorted = false;
     for (int c = threadIdx.x; c < npad / kChunkElems; c += TH) {
         const int k = c & 31, t = c >> 5;
         const int p0 = k * run + t * kChunkElems;
@@ -691,36 +738,53 @@ __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1)
             gc[4] = g1.x; gc[5] = g1.y; gc[6] = g1.z; gc[7] = g1.w;
         }
         uint32_t wv[kChunkElems / 2];
+        const uint32_t lanebit = 1u << k;
+        if (p0 + kChunkElems < n) {  // the row goes on after the chunk
 #pragma unroll
-        for (int j = 0; j < kChunkElems; ++j) {
-            const int p = p0 + j;
-            uint16_t e;
-            if (p < n) {
-                const bool step = (p == n - 1) || ((cp[j] >> ib) < (cp[j + 1] >> ib));
-                int word = (int)(cp[j] & imask);
-                if ((gc[j] >> k) & 1u) word = L.off_b + rot_b(word);
-                bad |= word >= L.words || word == n;
-                e = make_entry(word, step, j);
-            } else {
-                e = make_entry(n, false, j);
+            for (int j = 0; j < kChunkElems; ++j) {
+                const uint32_t i = cp[j] & imask;
+                const bool tob = (gc[j] & lanebit) != 0u;
+                const uint32_t word = tob ? (uint32_t)L.off_b + (uint32_t)rot_b((int)i) : i;
+                // words ascend, and two of one value differ below the value bits only
+                const uint32_t f = (cp[j] ^ cp[j + 1]) > imask ? (j & 1 ? 0x10000u : 0x8000u) : 0u;
+                unsorted |= cp[j] >= cp[j + 1];
+                // a sample index in range names a word of the weight array, and not the padding word
+                bad |= i >= (uint32_t)(tob ? L.nb : n);
+                if (j & 1) wv[j >> 1] |= (word << 17) | f;  // make_entry's two forms
+                else wv[j >> 1] = word | f;
             }
-            if (j & 1) wv[j >> 1] |= (uint32_t)e << 16;
-            else wv[j >> 1] = e;
+        } else {
+#pragma unroll
+            for (int j = 0; j < kChunkElems; ++j) {
+                const int p = p0 + j;
+                uint32_t e = make_entry(n, false, j);
+                if (p < n) {
+                    const uint32_t i = cp[j] & imask;
+                    const bool tob = (gc[j] & lanebit) != 0u;
+                    const bool last = p == n - 1;
+                    unsorted |= !last && cp[j] >= cp[j + 1];
+                    bad |= i >= (uint32_t)(tob ? L.nb : n);
+                    e = make_entry(tob ? L.off_b + rot_b((int)i) : (int)i, last || (cp[j] ^ cp[j + 1]) > imask, j);
+                }
+                if (j & 1) wv[j >> 1] |= e << 16;
+                else wv[j >> 1] = e;
+            }
         }
         reinterpret_cast<uint4 *>(out)[c] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+    }
+    if (__syncthreads_or(unsorted)) {  // the two-word sort writes the row again
+        if (threadIdx.x == 0) ovf[1 + atomicAdd(ovf, 1)] = (int32_t)blockIdx.x;
+        return;
     }
     row_written(bad, stat);
 }
 
 template <int IPT, int TH>
 static size_t sort_packed_smem() {
-    constexpr bool RS = packed_ranks_in_smem(IPT, TH);
-    const size_t hist = (size_t)kPkRadix * (TH / 32 + 1) * (RS ? 2 : 4);
-    return (size_t)TH * IPT * 4 + (RS ? (size_t)TH * IPT * 2 : 0) + ((hist + 15) & ~(size_t)15) +
-           (size_t)(TH * IPT / 32 + TH / 32 + 2) * 4;
+    return (size_t)(TH * IPT + kPkRadix + kPkRadix * (TH / 32) + TH * IPT / 32 + kPkRadix / 32 + 2 * (TH / 32) + 32) * 4;
 }
 
-template <int IPT, int TH = kPkThreads>
+template <int IPT, int TH>
 static cudaError_t launch_sort_packed(const int32_t *ii_t, const uint16_t *ii16, int ii_stride, int w,
                                       const DevFeature *feat,
                                       int64_t f0, int64_t nf, const WeightLayout &L, uint16_t *rows,
@@ -749,9 +813,9 @@ static cudaError_t launch_sort_wide(const int32_t *ii_t, int ii_stride, int w, c
 #undef VJB_SORT_CASE
 }
 
-// Rows of a tile: the packed sort for every row (512 threads up to 16,384
-// samples, 1024 above), then the two-word sort for the rows whose value span
-// and sample index do not fit one word, which the packed sort lists.
+// Rows of a tile: the packed sort for every row, then the two-word sort for
+// the rows that the packed sort lists: those whose value span and sample index
+// do not fit one word (and any it would have written out of order).
 // `ii16` (the integral images modulo 2^16, or null) serves the packed sort's
 // features of small boxes.  `scratch` (3 + nf ints of device memory): [0] and [1] the table's check
 // state (see row_written; zeroed by the caller once per table), [2] the
@@ -765,29 +829,32 @@ cudaError_t launch_sort_rows(const int32_t *ii_t, const uint16_t *ii16, int ii_s
     int32_t *stat = scratch, *ovf = scratch + 2;
     cudaError_t e = cudaMemsetAsync(ovf, 0, sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
-    if (n <= kPkThreads * 32) {
-#define VJB_PK_CASE(I) launch_sort_packed<I>(ii_t, ii16, ii_stride, w, feat, f0, nf, L, rows, npad, ovf, stat, st)
-        const int ipt = (n + kPkThreads - 1) / kPkThreads;
-        if (ipt <= 4) e = VJB_PK_CASE(4);
-        else if (ipt <= 8) e = VJB_PK_CASE(8);
-        else if (ipt <= 12) e = VJB_PK_CASE(12);
-        else if (ipt <= 16) e = VJB_PK_CASE(16);
-        else if (ipt <= 20) e = VJB_PK_CASE(20);
-        else if (ipt <= 24) e = VJB_PK_CASE(24);
-        else if (ipt <= 28) e = VJB_PK_CASE(28);
-        else if (ipt <= 30) e = VJB_PK_CASE(30);
-        else e = VJB_PK_CASE(32);
+    // the variant with the fewest idle items: TH threads of I items
+#define VJB_PK_CASE(I, TH) \
+    if (n <= (I) * (TH))   \
+        e = launch_sort_packed<I, TH>(ii_t, ii16, ii_stride, w, feat, f0, nf, L, rows, npad, ovf, stat, st); \
+    else
+    VJB_PK_CASE(8, 128)
+    VJB_PK_CASE(16, 128)
+    VJB_PK_CASE(24, 128)
+    VJB_PK_CASE(32, 128)
+    VJB_PK_CASE(20, 256)
+    VJB_PK_CASE(24, 256)
+    VJB_PK_CASE(28, 256)
+    VJB_PK_CASE(32, 256)
+    VJB_PK_CASE(20, 512)
+    VJB_PK_CASE(24, 512)
+    VJB_PK_CASE(28, 512)
+    VJB_PK_CASE(30, 512)
+    VJB_PK_CASE(32, 512)
+    VJB_PK_CASE(28, 640)
+    VJB_PK_CASE(30, 640)
+    VJB_PK_CASE(32, 640)
+    VJB_PK_CASE(24, 1024)
+    VJB_PK_CASE(28, 1024)
+    VJB_PK_CASE(32, 1024)
+    e = cudaErrorInvalidValue;
 #undef VJB_PK_CASE
-    } else {
-#define VJB_PK_WIDE(I) \
-    launch_sort_packed<I, 1024>(ii_t, ii16, ii_stride, w, feat, f0, nf, L, rows, npad, ovf, stat, st)
-        const int ipt = (n + 1023) / 1024;
-        if (ipt <= 20) e = VJB_PK_WIDE(20);
-        else if (ipt <= 24) e = VJB_PK_WIDE(24);
-        else if (ipt <= 28) e = VJB_PK_WIDE(28);
-        else e = VJB_PK_WIDE(32);
-#undef VJB_PK_WIDE
-    }
     if (e != cudaSuccess) return e;
     int32_t count = 0;
     e = cudaMemcpyAsync(&count, ovf, sizeof(int32_t), cudaMemcpyDeviceToHost, st);

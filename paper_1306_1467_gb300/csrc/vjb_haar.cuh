@@ -46,35 +46,44 @@ __device__ __forceinline__ int32_t haar_value(const int32_t *__restrict__ ii_t, 
     }
 }
 
-// The combination of haar_value for four windows at once, from a loader that
-// returns the four windows' integral-image values at point (px, py).
-template <class Load4>
-__device__ __forceinline__ int4 haar_combine4(int type, int x, int y, int fw, int fh, Load4 P) {
-    auto add = [](int4 a, int4 b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
-    auto sub = [](int4 a, int4 b) { return make_int4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); };
-    auto R = [&](int rx, int ry, int rw, int rh) {
-        return sub(add(P(rx + rw, ry + rh), P(rx, ry)), add(P(rx + rw, ry), P(rx, ry + rh)));
-    };
+// A feature's value as sums of integral-image points: the points added and
+// those subtracted (`pos`, `neg`), from a loader P(px, py) of the points and
+// an adder.  With C0, C1, ... the point columns (or rows) at the rectangles'
+// edges, two rectangles give C0 - 2 C1 + C2 and three C0 - 2 C1 + 2 C2 - C3,
+// bottom minus top (right minus left); four give -(x) (y) of two such pairs.
+template <class V, class Load, class Add>
+__device__ __forceinline__ void haar_sums(int type, int x, int y, int fw, int fh, Load P, Add add, V &pos, V &neg) {
+    auto twice = [&](V a) { return add(a, a); };
     switch (type) {
     case VJB_HAAR_2H: {
-        const int a = fw >> 1;
-        return sub(R(x + a, y, a, fh), R(x, y, a, fh));
+        const int a = fw >> 1, b = y + fh;
+        pos = add(add(P(x, b), P(x + fw, b)), twice(P(x + a, y)));
+        neg = add(add(P(x, y), P(x + fw, y)), twice(P(x + a, b)));
+        break;
     }
     case VJB_HAAR_2V: {
-        const int b = fh >> 1;
-        return sub(R(x, y + b, fw, b), R(x, y, fw, b));
+        const int a = fh >> 1, r = x + fw;
+        pos = add(add(P(r, y), P(r, y + fh)), twice(P(x, y + a)));
+        neg = add(add(P(x, y), P(x, y + fh)), twice(P(r, y + a)));
+        break;
     }
     case VJB_HAAR_3H: {
-        const int a = fw / 3;
-        return sub(sub(R(x + a, y, a, fh), R(x, y, a, fh)), R(x + 2 * a, y, a, fh));
+        const int a = fw / 3, b = y + fh;
+        pos = add(add(P(x, b), P(x + fw, y)), twice(add(P(x + 2 * a, b), P(x + a, y))));
+        neg = add(add(P(x, y), P(x + fw, b)), twice(add(P(x + 2 * a, y), P(x + a, b))));
+        break;
     }
     case VJB_HAAR_3V: {
-        const int b = fh / 3;
-        return sub(sub(R(x, y + b, fw, b), R(x, y, fw, b)), R(x, y + 2 * b, fw, b));
+        const int a = fh / 3, r = x + fw;
+        pos = add(add(P(r, y), P(x, y + fh)), twice(add(P(r, y + 2 * a), P(x, y + a))));
+        neg = add(add(P(x, y), P(r, y + fh)), twice(add(P(x, y + 2 * a), P(r, y + a))));
+        break;
     }
     default: {
-        const int a = fw >> 1, b = fh >> 1;
-        return sub(add(R(x + a, y, a, b), R(x, y + b, a, b)), add(R(x, y, a, b), R(x + a, y + b, a, b)));
+        const int a = fw >> 1, b = fh >> 1, r = x + fw, t = y + fh;
+        pos = twice(add(add(P(x + a, y), P(x + a, t)), add(P(x, y + b), P(r, y + b))));
+        neg = add(add(add(P(x, y), P(r, y)), add(P(x, t), P(r, t))), twice(twice(P(x + a, y + b))));
+        break;
     }
     }
 }
@@ -84,9 +93,12 @@ __device__ __forceinline__ int4 haar_combine4(int type, int x, int y, int fw, in
 __device__ __forceinline__ int4 haar_value4(const int32_t *__restrict__ ii_t, int stride, int w, int type,
                                             int x, int y, int fw, int fh, int i) {
     const int W1 = w + 1;
-    return haar_combine4(type, x, y, fw, fh, [&](int px, int py) -> int4 {
-        return __ldg(reinterpret_cast<const int4 *>(ii_t + (size_t)(py * W1 + px) * stride + i));
-    });
+    int4 p, q;
+    haar_sums<int4>(
+        type, x, y, fw, fh,
+        [&](int px, int py) { return __ldg(reinterpret_cast<const int4 *>(ii_t + (size_t)(py * W1 + px) * stride + i)); },
+        [](int4 a, int4 b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }, p, q);
+    return make_int4(p.x - q.x, p.y - q.y, p.z - q.z, p.w - q.w);
 }
 
 // Area of a feature's subtracted rectangles: its value lies in
@@ -104,20 +116,30 @@ __device__ __forceinline__ int haar_neg_area(int type, int fw, int fh) {
 // 65535.
 constexpr int kNarrowArea = 257;
 
-// haar_value4 for a feature with fw * fh <= kNarrowArea from the integral
-// images modulo 2^16 (ii16, same layout): one 8-byte load per corner.  The
-// corner combination is exact modulo 2^16, and the value is the one integer
-// of its residue class in [-255 * neg, -255 * neg + 65535].
-__device__ __forceinline__ int4 haar_value4_narrow(const uint16_t *__restrict__ ii16, int stride, int w,
-                                                   int type, int x, int y, int fw, int fh, int i) {
+// Two 16-bit sums in one word.
+__device__ __forceinline__ uint32_t add16x2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("add.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
+// A feature with fw * fh <= kNarrowArea on the four windows i .. i + 3 (i and
+// the row stride multiples of 4) from the integral images modulo 2^16 (ii16,
+// same layout): one 8-byte load per corner, two windows to a word.  The corner
+// combination is exact modulo 2^16, and the value is the one integer of its
+// residue class in [-255 * neg, -255 * neg + 65535]; returned are the four
+// values' offsets from the lower end of that range, 16 bits each.
+__device__ __forceinline__ uint2 haar_offsets4(const uint16_t *__restrict__ ii16, int stride, int w, int type,
+                                               int x, int y, int fw, int fh, int i) {
     const int W1 = w + 1;
-    const int4 r = haar_combine4(type, x, y, fw, fh, [&](int px, int py) -> int4 {
-        const uint2 q = __ldg(reinterpret_cast<const uint2 *>(ii16 + (size_t)(py * W1 + px) * stride + i));
-        return make_int4((int)(q.x & 0xffffu), (int)(q.x >> 16), (int)(q.y & 0xffffu), (int)(q.y >> 16));
-    });
-    const int lo = -255 * haar_neg_area(type, fw, fh);
-    auto lift = [lo](int v) { return lo + (int)((uint32_t)(v - lo) & 0xffffu); };
-    return make_int4(lift(r.x), lift(r.y), lift(r.z), lift(r.w));
+    uint2 p, q;
+    haar_sums<uint2>(
+        type, x, y, fw, fh,
+        [&](int px, int py) { return __ldg(reinterpret_cast<const uint2 *>(ii16 + (size_t)(py * W1 + px) * stride + i)); },
+        [](uint2 a, uint2 b) { return make_uint2(add16x2(a.x, b.x), add16x2(a.y, b.y)); }, p, q);
+    // p - q + 255 neg, the subtraction as ~q + 1
+    const uint32_t up = ((uint32_t)(255 * haar_neg_area(type, fw, fh) + 1) & 0xffffu) * 0x10001u;
+    return make_uint2(add16x2(add16x2(p.x, up), ~q.x), add16x2(add16x2(p.y, up), ~q.y));
 }
 
 }  // namespace vjb
