@@ -428,8 +428,7 @@ static cudaError_t launch_sort_ipt(const int32_t *ii_t, int ii_stride, int w, co
 //
 // Threads per CTA grow with the row (128 up to 4,096 samples, 256 up to 8,192,
 // 512 up to 16,384), 1,024 threads an SM in all: small CTAs leave other rows
-// to run while one waits at a barrier (24x24 / 2,003 in 512-thread CTAs: twice
-// the time).  From 16,385 to 20,480 samples two CTAs of 640 threads still fit
+// to run while one waits at a barrier.  From 16,385 to 20,480 samples two CTAs of 640 threads still fit
 // an SM (18,300: 26.0 ms, 29.9 with one CTA of 1,024); above, one of 1,024.
 //
 // Measured and dropped: one pass with a counter per value for spans up to 14

@@ -405,51 +405,70 @@ constexpr int kNoAllocDone = 2 * kNoAllocMaxCtas;      // completion counter
 constexpr int kNoAllocFlags = 2 * kNoAllocMaxCtas + 1; // error flags of the call
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kNoAllocWords];
 
+// Stage of the caller's table: 16 lines, 1,024 entries of the value order.
+// Lane l takes half a line, 32 neighbouring entries.
+constexpr int kNoAllocLines = 16;
+constexpr int kNoAllocStage = kNoAllocLines * kLineBytes;
+// The weights take the whole 15-bit index range, zero from n on, so that an
+// entry above n reads as padding without a clamp at every gather.
+constexpr int kNoAllocWeights = 32768;
+
 // Dynamic shared memory of k_screen_noalloc: the TMA rings first (1 KiB
-// aligned), then the n + 1 weights, the mbarriers and the per-warp minima.
-static size_t noalloc_smem_bytes(const SearchShape &s, int n) {
+// aligned), then the weights, the mbarriers and the per-warp minima.
+static size_t noalloc_smem_bytes(const SearchShape &s) {
     size_t b = 1024;
-    b += (size_t)s.warps * s.stages * kStageBytes;
-    b += align_up((size_t)(n + 1) * 4, 16);
+    b += (size_t)s.warps * s.stages * kNoAllocStage;
+    b += (size_t)kNoAllocWeights * 4;
     b += (size_t)s.warps * s.stages * 8;
     b += (size_t)s.warps * 4;
     return b;
 }
 
-// Same unit as screen_unit, with every gathered index clamped to n: the table
-// comes straight from the caller, so an entry above n reads as padding.
-__device__ __forceinline__ void screen_unit_clamped(uint32_t sbase, int unit, int lane,
-                                                    int lines_here, uint32_t n,
-                                                    const float *__restrict__ sv, float &chi,
-                                                    float &clo, float &MX, float &MN) {
-    const uint32_t line = (uint32_t)unit * 8u + ((uint32_t)lane >> 2);
-    const uint32_t sw = ((uint32_t)lane >> 2) & 7u;
-    const uint32_t c0 = ((2u * ((uint32_t)lane & 3u)) ^ sw) << 4;
-    const uint32_t c1 = ((2u * ((uint32_t)lane & 3u) + 1u) ^ sw) << 4;
-    const uint32_t pad2 = n | (n << 16);
-    uint4 q0 = make_uint4(pad2, pad2, pad2, pad2), q1 = q0;
-    if (line < (uint32_t)lines_here) {
-        q0 = lds128(sbase + line * kLineBytes + c0);
-        q1 = lds128(sbase + line * kLineBytes + c1);
-    }
-    const uint32_t wd[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
-    float g[16];
+// One stage of a row.  The lane's 32 entries are two pieces of 16 summed from
+// zero side by side; their largest and smallest prefixes at valid splits are
+// placed on the row by an FP32 scan of the 32 lanes' totals and the
+// compensated sum of the stages before (chi + clo).  Lines past the row's end
+// arrive as zeros: no flags, and their sums come after every split of the row.
+//
+// What bounds it: the shared-memory pipe (81% busy under ncu, ALU 53%).  The
+// caller's order is one random gather an entry, 3.5 wavefronts a warp
+// instruction, against 2 with the two bank-balanced copies of k_screen; with
+// the rest 4.4 wavefronts per 32 entries, 218 us at 16x16 / 15,000 if the pipe
+// never waited.  A scan per 1,024 entries instead of per 512, no clamps at the
+// gathers, the weights staged behind the first copies and 16 warps instead of
+// 8: 452 -> 281 us a call there (3.46 TB/s).  Weights first in shared memory
+// (constant gather addresses) were slower, 299 us.
+__device__ __forceinline__ void screen_stage_plain(uint32_t sbase, int lane, const float *__restrict__ sv, float &chi,
+                                                   float &clo, float &MX, float &MN) {
+    // chunk c of line l is stored at chunk c ^ (l mod 8) (128-byte swizzle):
+    // eight lanes (four lines) cover all the banks
+    const uint32_t line = (uint32_t)lane >> 1, first = ((uint32_t)lane & 1u) * 4u;
+    const uint32_t at = sbase + line * kLineBytes;
+    uint32_t w[2][8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        g[2 * j] = sv[min(wd[j] & kIndexMask, n)];
-        g[2 * j + 1] = sv[min((wd[j] >> 16) & kIndexMask, n)];
+    for (int c = 0; c < 4; ++c) {
+        const uint4 q = lds128(at + (((first + c) ^ (line & 7u)) << 4));
+        uint32_t *x = w[c >> 1] + 4 * (c & 1);
+        x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
     }
-    float a = 0.f, mx = -INFINITY, mn = INFINITY;
+    float g[2][16];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        a += g[j];
-        const uint32_t fl = (j & 1) ? (wd[j >> 1] & 0x80000000u) : (wd[j >> 1] & 0x8000u);
-        if (fl) {
-            mx = fmaxf(mx, a);
-            mn = fminf(mn, a);
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            g[u][2 * j] = sv[w[u][j] & kIndexMask];
+            g[u][2 * j + 1] = sv[(w[u][j] >> 16) & kIndexMask];
         }
-    }
-    float x = a;
+    float a[2] = {0.f, 0.f}, mx[2] = {-INFINITY, -INFINITY}, mn[2] = {INFINITY, INFINITY};
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            a[u] += g[u][j];
+            minmax_if(w[u][j >> 1] & ((j & 1) ? 0x80000000u : 0x8000u), a[u], mx[u], mn[u]);
+        }
+    const float own = a[0] + a[1];
+    float x = own;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const float y = __shfl_up_sync(0xffffffffu, x, d);
@@ -457,12 +476,11 @@ __device__ __forceinline__ void screen_unit_clamped(uint32_t sbase, int unit, in
     }
     float excl = __shfl_up_sync(0xffffffffu, x, 1);
     if (lane == 0) excl = 0.f;
-    const float tot = __shfl_sync(0xffffffffu, x, 31);
-    const float base = chi + (clo + excl);
-    MX = fmaxf(MX, base + mx);
-    MN = fminf(MN, base + mn);
+    const float b0 = chi + (clo + excl), b1 = chi + (clo + (excl + a[0]));
+    MX = fmaxf(MX, fmaxf(b0 + mx[0], b1 + mx[1]));
+    MN = fminf(MN, fminf(b0 + mn[0], b1 + mn[1]));
     float s, e;
-    two_sum(chi, tot, s, e);
+    two_sum(chi, __shfl_sync(0xffffffffu, x, 31), s, e);
     chi = s;
     clo += e;
 }
@@ -477,20 +495,24 @@ __global__ void __launch_bounds__(512, 1)
     const int nw = blockDim.x >> 5;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *rings = base;
-    float *sv = reinterpret_cast<float *>(rings + (size_t)nw * stages * kStageBytes);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sv + align_up((size_t)(n + 1), 4));
+    float *sv = reinterpret_cast<float *>(rings + (size_t)nw * stages * kNoAllocStage);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sv + kNoAllocWeights);
     float *wbest = reinterpret_cast<float *>(bars + nw * stages);
     __shared__ int32_t wfeat[16];
     __shared__ bool last_cta;
 
-    for (int i = threadIdx.x; i <= n; i += blockDim.x) sv[i] = (i < n) ? v[i] : 0.f;
-    const uint32_t ring_w = smem_u32(rings + (size_t)warp * stages * kStageBytes);
+    const uint32_t ring_w = smem_u32(rings + (size_t)warp * stages * kNoAllocStage);
     const uint32_t bar_w = smem_u32(bars + warp * stages);
     if (lane == 0) {
         for (int s = 0; s < stages; ++s) mbar_init(bar_w + 8 * s, 1);
         fence_barrier_init();
     }
-    __syncthreads();
+    // rows shorter than a stage: the lines no copy writes hold zeros, as the
+    // lines past a longer row's end do
+    for (int s = 0; s < stages; ++s)
+        for (int i = box_lines * kLineBytes + 16 * lane; i < kNoAllocStage; i += 16 * 32)
+            *reinterpret_cast<uint4 *>(rings + (size_t)(warp * stages + s) * kNoAllocStage + i) = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
 
     const int64_t gw = (int64_t)blockIdx.x * nw + warp;
     const int64_t G = (int64_t)gridDim.x * nw;
@@ -498,51 +520,52 @@ __global__ void __launch_bounds__(512, 1)
     const int nc = (lines_per_row + box_lines - 1) / box_lines;
     const int64_t total = nf_w * nc;
     const uint32_t tx = (uint32_t)box_lines * kLineBytes;
-    auto issue = [&](int64_t seq) {
-        const int64_t k = seq / nc;
-        const int c = (int)(seq - k * nc);
-        const int64_t f = gw + k * G;
-        const int stage = (int)(seq % stages);
-        const uint32_t bar = bar_w + 8u * stage;
+    // producer (lane 0): the next stage to load, in this warp's order
+    int64_t issued = 0, prow = gw;
+    int pline = 0, pstage = 0;
+    auto issue_next = [&]() {
+        if (issued >= total) return;
+        const uint32_t bar = bar_w + 8u * (uint32_t)pstage;
         mbar_arrive_expect_tx(bar, tx);
-        tma_load_3d(ring_w + (uint32_t)stage * kStageBytes, &tmap, 0, c * box_lines, (int32_t)f, bar);
+        tma_load_3d(ring_w + (uint32_t)pstage * kNoAllocStage, &tmap, 0, pline, (int32_t)prow, bar);
+        pline += box_lines;
+        if (pline >= lines_per_row) { pline = 0; prow += G; }
+        if (++pstage == stages) pstage = 0;
+        ++issued;
     };
-    if (lane == 0) {
-        const int64_t pro = total < stages ? total : stages;
-        for (int64_t s = 0; s < pro; ++s) issue(s);
-    }
+    if (lane == 0)
+        for (int s = 0; s < stages; ++s) issue_next();
     __syncwarp();
+    // the weights, staged while the first copies are in flight
+    for (int i = threadIdx.x; i < kNoAllocWeights; i += blockDim.x) sv[i] = i < n ? v[i] : 0.f;
+    __syncthreads();
 
     float best = INFINITY;
     int32_t bestf = 0x7fffffff;
-    int64_t seq = 0;
+    int64_t consumed = 0;
+    int cstage = 0;
+    uint32_t cpar = 0;
     bool ok = true;
     for (int64_t k = 0; k < nf_w && ok; ++k) {
         const int64_t f = gw + k * G;
         float chi = 0.f, clo = 0.f, MX = 0.f, MN = 0.f;
         for (int c = 0; c < nc; ++c) {
-            const int stage = (int)(seq % stages);
-            const uint32_t par = (uint32_t)((seq / stages) & 1);
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar_w + 8u * stage, par))) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar_w + 8u * (uint32_t)cstage, cpar))) {
                 ok = false;
                 break;
             }
-            const int lines_here = min(box_lines, lines_per_row - c * box_lines);
-            const int units = (lines_here + 7) >> 3;
-            const uint32_t sbase = ring_w + (uint32_t)stage * kStageBytes;
-            for (int u = 0; u < units; ++u)
-                screen_unit_clamped(sbase, u, lane, lines_here, (uint32_t)n, sv, chi, clo, MX, MN);
+            screen_stage_plain(ring_w + (uint32_t)cstage * kNoAllocStage, lane, sv, chi, clo, MX, MN);
             __syncwarp();
-            if (lane == 0 && seq + stages < total) {
+            if (lane == 0) {
                 fence_proxy_async_smem();
-                issue(seq + stages);
+                issue_next();
             }
-            ++seq;
+            if (++cstage == stages) { cstage = 0; cpar ^= 1u; }
+            ++consumed;
         }
         if (!ok) break;
-        MX = warp_max(MX);
-        MN = warp_min(MN);
-        const float e = fminf(Tp - MX, Tm + MN);
+        // (a min does not round: the least of the lanes' errors is the row's)
+        const float e = float_from_order_key(__reduce_min_sync(0xffffffffu, float_order_key(fminf(Tp - MX, Tm + MN))));
         if (lane == 0) {
             ferr[f] = e;
             if (e < best) { best = e; bestf = (int32_t)f; }
@@ -550,9 +573,10 @@ __global__ void __launch_bounds__(512, 1)
     }
     if (!ok && lane == 0) {
         atomicOr(&scratch[kNoAllocFlags], (uint32_t)kFlagWaitTimeout);
-        const int64_t issued = (seq + stages < total) ? seq + stages : total;
-        for (int64_t s = seq; s < issued; ++s)
-            mbar_wait_bounded(bar_w + 8u * (uint32_t)(s % stages), (uint32_t)((s / stages) & 1), 100000000ull);
+        for (const int64_t pending = issued; consumed < pending; ++consumed) {
+            mbar_wait_bounded(bar_w + 8u * (uint32_t)cstage, cpar, 100000000ull);
+            if (++cstage == stages) { cstage = 0; cpar ^= 1u; }
+        }
     }
     __syncwarp();
     if (lane == 0) { wbest[warp] = best; wfeat[warp] = bestf; }
@@ -664,14 +688,13 @@ extern "C" int vjb_screen_noalloc(const uint16_t *rows, const float *v, int32_t 
         }
     }
     const int grid = ctas ? ctas : std::min(D.num_sms, kNoAllocMaxCtas);
-    const SearchShape tries[] = {{8, 4, 1, 1, 32}, {8, 3, 1, 1, 32}, {4, 4, 1, 1, 32}, {4, 2, 1, 1, 32},
-                                 {2, 2, 1, 1, 32}};
+    const SearchShape tries[] = {{16, 3, 1, 1, kNoAllocLines}, {16, 2, 1, 1, kNoAllocLines}, {8, 2, 1, 1, kNoAllocLines}};
     const SearchShape *shape = nullptr;
     for (const auto &s : tries)
-        if (noalloc_smem_bytes(s, n) <= (size_t)D.max_smem) { shape = &s; break; }
-    if (!shape) return report_error(VJB_EINVAL, "vjb_screen_noalloc: n too large for shared memory");
+        if (noalloc_smem_bytes(s) <= (size_t)D.max_smem) { shape = &s; break; }
+    if (!shape) return report_error(VJB_EINVAL, "vjb_screen_noalloc: the weights do not fit shared memory");
     const int lines = npad / kLineElems;
-    const int box_lines = std::min(kBoxLinesMax, lines);
+    const int box_lines = std::min(kNoAllocLines, lines);
     CUtensorMap tmap;
     cuuint64_t dims[3] = {(cuuint64_t)kLineElems, (cuuint64_t)lines, (cuuint64_t)nfeat};
     cuuint64_t strides[2] = {(cuuint64_t)kLineBytes, (cuuint64_t)lines * kLineBytes};
@@ -685,7 +708,7 @@ extern "C" int vjb_screen_noalloc(const uint16_t *rows, const float *v, int32_t 
     // the counter and the flags must start at zero; the partials are all overwritten
     if (cudaMemsetAsync(D.scratch + kNoAllocDone, 0, 2 * sizeof(uint32_t), st) != cudaSuccess)
         return report_error(VJB_ECUDA, "vjb_screen_noalloc: clearing the scratch counter failed");
-    k_screen_noalloc<<<grid, shape->warps * 32, noalloc_smem_bytes(*shape, n), st>>>(
+    k_screen_noalloc<<<grid, shape->warps * 32, noalloc_smem_bytes(*shape), st>>>(
         tmap, v, n, lines, box_lines, nfeat, shape->stages, (float)t_pos, (float)t_neg, feature_err,
         best_err, best_feature, D.scratch);
     const cudaError_t e = cudaGetLastError();
