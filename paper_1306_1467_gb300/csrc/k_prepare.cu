@@ -8,44 +8,74 @@
 
 #include "vjb_device.cuh"
 #include "vjb_haar.cuh"
+#include "vjb_integral.cuh"
 #include "vjb_internal.cuh"
 
 namespace vjb {
 
 // ---- K1: integral images --------------------------------------------------------
-// One thread per window.  Output is point-major, ii_t[(y * (w + 1) + x) * stride + i],
-// so that the feature kernel reads consecutive windows with coalesced loads.
-// ii(x, y) = sum of pixels with x' < x and y' < y (zero first row and column),
-// built row by row: ii(x, y) = ii(x, y - 1) + (sum of row y - 1 up to x - 1).
-// With ii16 non-null, also the values modulo 2^16 in the same layout (the
-// sort evaluates features of small boxes from these).
-__global__ void k_integral(const uint8_t *__restrict__ px, int n, int h, int w,
-                           int32_t *__restrict__ ii_t, uint16_t *__restrict__ ii16, int stride) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// A CTA takes 32 windows, a lane each.  Output is point-major, ii_t[(y * (w + 1) +
+// x) * stride + i], so that the feature kernels read consecutive windows with
+// coalesced loads.  ii(x, y) = sum of pixels with x' < x and y' < y (zero first
+// row and column): running sums along the rows in shared memory, then down the
+// columns, a band of rows at a time (the whole window where it fits).
+// ii16 receives the values modulo 2^16 in the same layout (the sort evaluates
+// features of small boxes from these).
+//
+// Bound by its writes for large sets and by the two chains of additions (w and
+// h long) for small ones: 10 us at 24x24 / 1,000 (ncu).  One thread per window,
+// each pixel after the one above it in memory, took 41 us there and 46 us at
+// 15,000.
+constexpr int kIntegralThreads = 512;
+
+__global__ void __launch_bounds__(kIntegralThreads)
+    k_integral(const uint8_t *__restrict__ px, int n, int h, int w, int band, int32_t *__restrict__ ii_t,
+               uint16_t *__restrict__ ii16, int stride) {
+    extern __shared__ __align__(16) int32_t sums[];  // [band][w][32], then the carry [w][32], then the pixels
+    int32_t *carry = sums + (size_t)band * w * 32;
+    uint32_t *tile = reinterpret_cast<uint32_t *>(carry + w * 32);
+    const int tstride = tile_stride(band * w);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int i0 = blockIdx.x * kTileWindows, i = i0 + lane;
     const int W1 = w + 1;
-    const uint8_t *img = px + (size_t)i * h * w;
-    for (int x = 0; x <= w; ++x) {
-        ii_t[(size_t)x * stride + i] = 0;
-        if (ii16) ii16[(size_t)x * stride + i] = 0;
-    }
-    for (int y = 1; y <= h; ++y) {
-        ii_t[(size_t)(y * W1) * stride + i] = 0;
-        if (ii16) ii16[(size_t)(y * W1) * stride + i] = 0;
-        int32_t row = 0;
-        for (int x = 1; x <= w; ++x) {
-            row += img[(y - 1) * w + (x - 1)];
-            const int32_t up = ii_t[(size_t)((y - 1) * W1 + x) * stride + i];
-            ii_t[(size_t)(y * W1 + x) * stride + i] = up + row;
-            if (ii16) ii16[(size_t)(y * W1 + x) * stride + i] = (uint16_t)(up + row);
+    const bool in = i < n;
+    auto put = [&](int point, int32_t v) {
+        if (in) {
+            ii_t[(size_t)point * stride + i] = v;
+            if (ii16) ii16[(size_t)point * stride + i] = (uint16_t)v;
         }
+    };
+    for (int x = warp; x <= w; x += nw) put(x, 0);
+    for (int y = 1 + warp; y <= h; y += nw) put(y * W1, 0);
+    for (int x = warp; x < w; x += nw) carry[x * 32 + lane] = 0;
+    for (int y0 = 0; y0 < h; y0 += band) {
+        const int rows = min(band, h - y0);
+        stage_pixels(px, i0, n, h * w, y0 * w, rows * w, tile, tstride);
+        __syncthreads();
+        row_sums(tile, tstride, rows, w, sums, w);
+        __syncthreads();
+        for (int x = warp; x < w; x += nw) {
+            int32_t v = carry[x * 32 + lane];
+#pragma unroll 4
+            for (int y = 0; y < rows; ++y) {
+                v += sums[(y * w + x) * 32 + lane];
+                put((y0 + y + 1) * W1 + x + 1, v);
+            }
+            carry[x * 32 + lane] = v;
+        }
+        __syncthreads();
     }
 }
 
 cudaError_t launch_integral(const uint8_t *px, int n, int h, int w, int32_t *ii_t, uint16_t *ii16,
                             int ii_stride, cudaStream_t st) {
-    const int b = 128;
-    k_integral<<<(n + b - 1) / b, b, 0, st>>>(px, n, h, w, ii_t, ii16, ii_stride);
+    auto bytes = [&](int band) { return ((size_t)band * w * 32 + w * 32 + 32 * tile_stride(band * w)) * 4; };
+    int band = h;  // two CTAs an SM, or a row at a time (up to 255 pixels: 73 KB)
+    while (band > 1 && bytes(band) > 100 * 1024) --band;
+    cudaError_t e = cudaFuncSetAttribute(k_integral, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(band));
+    if (e != cudaSuccess) return e;
+    k_integral<<<(n + kTileWindows - 1) / kTileWindows, kIntegralThreads, bytes(band), st>>>(px, n, h, w, band, ii_t,
+                                                                                            ii16, ii_stride);
     return cudaGetLastError();
 }
 

@@ -480,6 +480,9 @@ void vjb_destroy(vjb_ctx *c) {
     if (c->stream) cudaStreamSynchronize(c->stream);
     c->free_all();
     c->free_events();
+    if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
+    for (auto ev : c->cls_ev)
+        if (ev) cudaEventDestroy(ev);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
 }
@@ -712,40 +715,88 @@ int vjb_classify(vjb_ctx *c, const uint8_t *pixels, int32_t n, const vjb_stump *
     if (n < 1 || n > (1 << 26)) return fail(VJB_EINVAL, "n = %d outside [1, 2^26]", n);
     if (T < 0) return fail(VJB_EINVAL, "T < 0");
     double half = 0.0;
+    std::vector<ClassStump> cs((size_t)std::max(T, 1));
     for (int t = 0; t < T; ++t) {
         const vjb_stump &s = stumps[t];
         if (s.feature < 0 || s.feature >= c->nfeat || (s.polarity != 1 && s.polarity != -1) || std::isnan(s.alpha))
             return fail(VJB_EINVAL, "stump %d is not a stump of this window size", t);
         half += s.alpha;
+        const vjb_feature &f = c->feats[(size_t)s.feature];
+        cs[(size_t)t] = ClassStump{DevFeature{f.type, f.x, f.y, f.w, f.h, 0, 0, 0}, s.threshold, s.polarity, s.alpha};
     }
     half *= 0.5;  // C(x) = 1 iff sum alpha_t h_t(x) >= 1/2 sum alpha_t
     int rc = set_dev(c);
     if (rc) return rc;
-    const size_t px_bytes = (size_t)n * c->h * c->w;
+    // Windows go to the device a part at a time, in two buffers, so that a part
+    // is classified while the next is copied (86 MB of 24x24 windows: the copy
+    // alone takes 490 us, the kernels 302; the call 831 us with parts of 24 MiB,
+    // 886 with 8 and 1,017 with 4, and 1,814 with one copy, integral images in
+    // memory and buffers allocated and freed).  Windows too large for shared
+    // memory go through integral images in memory, whole.
+    const size_t hw = (size_t)c->h * c->w;
+    const bool fused = classify_fits(c->h, c->w, c->max_smem);
+    const int part = fused ? (int)std::min<size_t>((size_t)(n + 31) / 32 * 32, std::max<size_t>(32, (kClassifyPartBytes / hw) / 32 * 32)) : n;
+    const int parts = (n + part - 1) / part;
     const int stride = (n + 31) / 32 * 32;
-    uint8_t *d_px = nullptr, *d_lab = nullptr;
-    int32_t *d_ii = nullptr;
-    vjb_stump *d_st = nullptr;
-    double *d_sc = nullptr;
-    auto cleanup = [&]() {
-        dfree(d_px); dfree(d_lab); dfree(d_ii); dfree(d_st); dfree(d_sc);
-    };
-    cudaError_t e = cudaMalloc(&d_px, px_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&d_ii, sizeof(int32_t) * (size_t)(c->h + 1) * (c->w + 1) * stride);
-    if (e == cudaSuccess) e = cudaMalloc(&d_lab, (size_t)n);
-    if (e == cudaSuccess) e = cudaMalloc(&d_st, sizeof(vjb_stump) * (size_t)std::max(T, 1));
-    if (e == cudaSuccess && scores) e = cudaMalloc(&d_sc, sizeof(double) * (size_t)n);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_px, pixels, px_bytes, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess && T > 0) e = cudaMemcpyAsync(d_st, stumps, sizeof(vjb_stump) * T, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = launch_integral(d_px, n, c->h, c->w, d_ii, nullptr, stride, c->stream);
-    if (e == cudaSuccess)
-        e = launch_strong_classify(d_ii, stride, n, c->w, c->d_feat, d_st, T, half, d_lab, d_sc, c->stream);
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t o_px1 = al(part * hw), o_st = o_px1 + (parts > 1 ? al(part * hw) : 0);
+    const size_t o_sc = o_st + al(sizeof(ClassStump) * cs.size()), o_lab = o_sc + (scores ? al(8 * (size_t)n) : 0);
+    const size_t o_ii = o_lab + al((size_t)n);
+    const size_t need = o_ii + (fused ? 0 : sizeof(int32_t) * (size_t)(c->h + 1) * (c->w + 1) * stride);
+    // kept with the context up to a bound: allocating and freeing cost a few
+    // microseconds, and for large calls hundreds
+    cudaError_t e = cudaSuccess;
+    if (need > c->cls_bytes) {
+        dfree(c->d_cls);
+        c->cls_bytes = 0;
+        e = cudaMalloc(&c->d_cls, need);
+        if (e == cudaSuccess) c->cls_bytes = need;
+    }
+    uint8_t *base = static_cast<uint8_t *>(c->d_cls);
+    uint8_t *d_lab = base + o_lab;
+    double *d_sc = scores ? reinterpret_cast<double *>(base + o_sc) : nullptr;
+    ClassStump *d_st = reinterpret_cast<ClassStump *>(base + o_st);
+    if (e == cudaSuccess && parts > 1 && !c->copy_stream) {
+        e = cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking);
+        for (auto &ev : c->cls_ev)
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess && T > 0) e = cudaMemcpyAsync(d_st, cs.data(), sizeof(ClassStump) * T, cudaMemcpyHostToDevice, c->stream);
+    for (int k = 0; k < parts && e == cudaSuccess; ++k) {
+        const int i0 = k * part, m = std::min(part, n - i0), buf = k & 1;
+        uint8_t *d_px = base + (buf ? o_px1 : 0);
+        cudaStream_t copies = parts > 1 ? c->copy_stream : c->stream;
+        // (buffer `buf` is free again once part k - 2 is classified)
+        if (k >= 2) e = cudaStreamWaitEvent(copies, c->cls_ev[2 + buf], 0);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d_px, pixels + i0 * hw, m * hw, cudaMemcpyHostToDevice, copies);
+        if (e == cudaSuccess && parts > 1) {
+            e = cudaEventRecord(c->cls_ev[buf], copies);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->cls_ev[buf], 0);
+        }
+        if (e != cudaSuccess) break;
+        if (fused) {
+            e = launch_classify_windows(d_px, m, c->h, c->w, d_st, T, half, d_lab + i0, d_sc ? d_sc + i0 : nullptr, c->stream);
+        } else {
+            int32_t *d_ii = reinterpret_cast<int32_t *>(base + o_ii);
+            e = launch_integral(d_px, n, c->h, c->w, d_ii, nullptr, stride, c->stream);
+            if (e == cudaSuccess) e = launch_strong_classify(d_ii, stride, n, c->w, d_st, T, half, d_lab, d_sc, c->stream);
+        }
+        c->launches += fused ? 1 : 2;
+        if (e == cudaSuccess && parts > 1) e = cudaEventRecord(c->cls_ev[2 + buf], c->stream);
+    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(labels, d_lab, (size_t)n, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess && scores)
         e = cudaMemcpyAsync(scores, d_sc, sizeof(double) * (size_t)n, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    c->launches += 2;
-    cleanup();
+    if (c->copy_stream) {
+        const cudaError_t e2 = cudaStreamSynchronize(c->copy_stream);
+        if (e == cudaSuccess) e = e2;
+    }
+    const cudaError_t e3 = cudaStreamSynchronize(c->stream);
+    if (e == cudaSuccess) e = e3;
+    if (c->cls_bytes > kClassifyKeepBytes) {
+        dfree(c->d_cls);
+        c->cls_bytes = 0;
+    }
     if (e != cudaSuccess)
         return fail(e == cudaErrorMemoryAllocation ? VJB_ENOMEM : VJB_ECUDA, "classify: %s", cudaGetErrorString(e));
     return VJB_OK;

@@ -54,6 +54,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 constexpr int kStageNone = 0, kStageLoaded = 1, kStageIntegral = 2, kStagePrepared = 3;
+constexpr size_t kClassifyPartBytes = 24u << 20;   // windows copied at a time
+constexpr size_t kClassifyKeepBytes = 64u << 20;  // largest workspace kept between calls
 constexpr int kRoundLaunches = 5;  // screen, shortlist, rescan, update a, update b
 
 using EventTriple = std::array<cudaEvent_t, 3>;  // round start, search end, round end
@@ -105,6 +107,13 @@ struct vjb_ctx {
     int stump_cap = 0;
     int bmin_cap = 0;
 
+    // vjb_classify: its workspace, the stream of its copies and their events
+    // (part copied, part classified; two of each)
+    void *d_cls = nullptr;
+    size_t cls_bytes = 0;
+    cudaStream_t copy_stream = nullptr;
+    cudaEvent_t cls_ev[4] = {nullptr, nullptr, nullptr, nullptr};
+
     std::vector<vjb_feature> feats;
     CUtensorMap tmap;
     bool tmap_ok = false;
@@ -139,7 +148,8 @@ struct vjb_ctx {
         rows_external = false;
         dfree(d_w); dfree(d_v); dfree(d_wtmp); dfree(d_ferr); dfree(d_bmin); dfree(d_cand);
         dfree(d_cand_ids); dfree(d_runres); dfree(d_cand_runs); dfree(d_miss); dfree(d_partials); dfree(d_scratch);
-        dfree(d_rs); dfree(d_stumps); dfree(d_last); dfree(d_diag);
+        dfree(d_rs); dfree(d_stumps); dfree(d_last); dfree(d_diag); dfree(d_cls);
+        cls_bytes = 0;
         stump_cap = bmin_cap = 0;
         feats.clear();
         stage = kStageNone;
