@@ -1,6 +1,6 @@
 // Weight kernels of a boosting round (Sec. 2.3):
 //  * k_init_weights: the initial weights of Table 2 (1/(2l) per face, 1/(2m)
-//    per non-face) or caller-given weights, normalised (step 1).  One CTA.
+//    per non-face) or caller-given weights, normalised (step 1).  One cluster.
 //  * k_update_a: the round's stump applied to every sample: e_i (misclassified
 //    or not) and FP64 partial sums of the misclassified and of all weight.
 //    The last CTA to finish forms the error (step 2, exact given the FP32
@@ -13,6 +13,7 @@
 //    the stored weights for the next search.
 // FP64 is used only for the sums, the error, beta, alpha and the one multiply
 // per sample of the renormalisation.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "vjb_device.cuh"
@@ -21,19 +22,35 @@
 
 namespace vjb {
 
-constexpr int kOneCta = 1024;
+// k_init_weights: 1,024 threads as a cluster of 8 CTAs on 8 SMs.  GB300's FP64
+// unit runs at a couple of lanes per clock per SM: one CTA of 1,024 threads
+// took 64 us for 1,000 samples (every warp of it added the 32 warps' sums, one
+// after another, five times) and 100 us for 15,000 (its own share of the FP64
+// work); this form takes 15 us at 15,000 (ncu), and
+// vjb_set_weights 107 -> 46 us there and 57 -> 26 us at 600.
+constexpr int kInitCtas = 8, kInitThreads = 128, kInitWarps = kInitThreads / 32;
 
-// Sum of one double per thread over the CTA (every thread gets the result,
-// added in a fixed order so that runs are reproducible).
-__device__ __forceinline__ double cta_sum(double x, double *red) {
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+// Sum of one double per thread over the cluster in a fixed order: lanes by a
+// butterfly, then the 32 warps' sums one after another.  `part` is this sum's
+// place in every CTA's shared memory, `total` where this CTA's threads find the
+// result; `adder` is the warp that adds up.
+__device__ __forceinline__ void cluster_partial(double x, double *part) {
     x = warp_sum_d(x);
-    __syncthreads();
-    if (lane == 0) red[wp] = x;
-    __syncthreads();
-    double s = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += red[k];
-    return s;
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = x;
+}
+__device__ __forceinline__ void cluster_total(double *part, double *all, double *total, int adder) {
+    if ((int)threadIdx.x >> 5 != adder) return;
+    const int lane = threadIdx.x & 31;
+    auto cluster = cooperative_groups::this_cluster();
+    static_assert(kInitCtas * kInitWarps == 32, "a lane per warp of the cluster");
+    all[lane] = cluster.map_shared_rank(part, lane / kInitWarps)[lane % kInitWarps];
+    __syncwarp();
+    if (lane == 0) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) s += all[k];
+        *total = s;
+    }
 }
 
 __device__ __forceinline__ void store_v(float *v, const WeightLayout &L, int i, float x) {
@@ -41,54 +58,60 @@ __device__ __forceinline__ void store_v(float *v, const WeightLayout &L, int i, 
     if (L.dual && i < L.nb) v[L.off_b + rot_b(i)] = x;
 }
 
-__global__ void __launch_bounds__(kOneCta)
-    k_init_weights(const uint8_t *__restrict__ y, WeightLayout L, const float *__restrict__ w_in,
+__global__ void __cluster_dims__(kInitCtas, 1, 1) __launch_bounds__(kInitThreads)
+    k_init_weights(const uint8_t *__restrict__ y, WeightLayout L, const float *__restrict__ w_in, double wf, double wn,
                    float *__restrict__ w, float *__restrict__ v, RoundState *rs) {
-    __shared__ double red[32];
-    const int n = L.n;
-    double l = 0.0, m = 0.0;
-    if (!w_in) {
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            if (y[i]) l += 1.0; else m += 1.0;
-        }
-        l = cta_sum(l, red);
-        m = cta_sum(m, red);
-    }
-    // Table 2: 1/(2l) for faces, 1/(2m) for non-faces
-    const double wf = w_in ? 0.0 : 1.0 / (2.0 * l), wn = w_in ? 0.0 : 1.0 / (2.0 * m);
+    __shared__ double part[3][kInitWarps], all[2][32], total[3];
+    auto cluster = cooperative_groups::this_cluster();
+    const int n = L.n, step = kInitCtas * kInitThreads, i0 = (int)(blockIdx.x * kInitThreads + threadIdx.x);
+    // caller-given weights, or Table 2's: wf = 1/(2l) for faces, wn = 1/(2m) for non-faces
     double tot = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x)
-        tot += w_in ? (double)w_in[i] : (y[i] ? wf : wn);
-    tot = cta_sum(tot, red);
-    const double r = 1.0 / tot;
+    for (int i = i0; i < n; i += step) tot += w_in ? (double)w_in[i] : (y[i] ? wf : wn);
+    cluster_partial(tot, part[0]);
+    cluster.sync();
+    cluster_total(part[0], all[0], &total[0], 0);
+    if (threadIdx.x == 0) total[1] = 1.0 / total[0];
+    __syncthreads();
+    tot = total[0];
+    const double r = total[1];
     double tp = 0.0, tn = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i = i0; i < n; i += step) {
         const double wi = w_in ? (double)w_in[i] : (y[i] ? wf : wn);
         const float f = __double2float_rn(wi * r);
         w[i] = f;
         store_v(v, L, i, y[i] ? f : -f);
         if (y[i]) tp += (double)f; else tn += (double)f;
     }
-    tp = cta_sum(tp, red);
-    tn = cta_sum(tn, red);
-    if (threadIdx.x == 0) {
-        v[n] = 0.f;
-        rs->t_pos = tp;
-        rs->t_neg = tn;
-        rs->weight_sum = tp + tn;
-        rs->status = VJB_OK;
-        rs->cand_count = 0;
-        rs->forced = 0;
-        rs->done_rescan = rs->done_update_a = rs->done_update_b = 0u;
-        rs->screen_min_bits = 0x7f800000u;
-        rs->in_round = 0;
-        if (!(tot > 0.0) || !isfinite(tot)) rs->flags |= kFlagBadWeights;
+    cluster_partial(tp, part[1]);
+    cluster_partial(tn, part[2]);
+    cluster.sync();
+    if (blockIdx.x == 0) {
+        cluster_total(part[1], all[0], &total[1], 0);
+        cluster_total(part[2], all[1], &total[2], 1);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            tp = total[1];
+            tn = total[2];
+            v[n] = 0.f;
+            rs->t_pos = tp;
+            rs->t_neg = tn;
+            rs->weight_sum = tp + tn;
+            rs->status = VJB_OK;
+            rs->cand_count = 0;
+            rs->forced = 0;
+            rs->done_rescan = rs->done_update_a = rs->done_update_b = 0u;
+            rs->screen_min_bits = 0x7f800000u;
+            rs->in_round = 0;
+            if (!(tot > 0.0) || !isfinite(tot)) rs->flags |= kFlagBadWeights;
+        }
     }
+    cluster.sync();  // no CTA leaves while another reads its shared memory
 }
 
-cudaError_t launch_init_weights(const uint8_t *y, const WeightLayout &L, const float *w_in,
+cudaError_t launch_init_weights(const uint8_t *y, int faces, const WeightLayout &L, const float *w_in,
                                 float *w, float *v, RoundState *rs, cudaStream_t st) {
-    k_init_weights<<<1, kOneCta, 0, st>>>(y, L, w_in, w, v, rs);
+    const double wf = 1.0 / (2.0 * faces), wn = 1.0 / (2.0 * (L.n - faces));
+    k_init_weights<<<kInitCtas, kInitThreads, 0, st>>>(y, L, w_in, wf, wn, w, v, rs);
     return cudaGetLastError();
 }
 

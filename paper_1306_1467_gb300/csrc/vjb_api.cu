@@ -318,6 +318,7 @@ int load_common(vjb_ctx *c, const uint8_t *pixels, const uint8_t *labels, int32_
     }
     rc = validate_labels(hy.data(), n);
     if (rc) return rc;
+    const int faces = (int)std::count(hy.begin(), hy.end(), (uint8_t)1);
     CK(cudaStreamSynchronize(c->stream));
     const bool same_shape = c->d_px && c->n == n && c->h == h && c->w == w;
     if (!same_shape) {
@@ -347,7 +348,7 @@ int load_common(vjb_ctx *c, const uint8_t *pixels, const uint8_t *labels, int32_
     CK(cudaMemcpyAsync(c->d_y, hy.data(), (size_t)n, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemsetAsync(c->d_rs, 0, sizeof(RoundState), c->stream));
     CK(cudaMemsetAsync(c->d_last, 0, sizeof(vjb_stump), c->stream));
-    CK(launch_init_weights(c->d_y, c->lay, nullptr, c->d_w, c->d_v, c->d_rs, c->stream));
+    CK(launch_init_weights(c->d_y, faces, c->lay, nullptr, c->d_w, c->d_v, c->d_rs, c->stream));
     c->launches += 1;
     CK(cudaStreamSynchronize(c->stream));
     c->stage = kStageLoaded;
@@ -637,7 +638,7 @@ int vjb_set_weights(vjb_ctx *c, const float *wts) {
     int rc = set_dev(c);
     if (rc) return rc;
     CK(cudaMemcpyAsync(c->d_wtmp, wts, sizeof(float) * c->n, cudaMemcpyHostToDevice, c->stream));
-    CK(launch_init_weights(c->d_y, c->lay, c->d_wtmp, c->d_w, c->d_v, c->d_rs, c->stream));
+    CK(launch_init_weights(c->d_y, 0, c->lay, c->d_wtmp, c->d_w, c->d_v, c->d_rs, c->stream));
     c->launches += 1;
     CK(cudaStreamSynchronize(c->stream));
     return VJB_OK;

@@ -226,7 +226,8 @@ cudaError_t launch_feature_values(const int32_t *ii_t, int ii_stride, int n, int
 cudaError_t launch_sort_rows(const int32_t *ii_t, const uint16_t *ii16, int ii_stride, int w,
                              const DevFeature *feat, int64_t f0, int64_t nf, const WeightLayout &L, uint16_t *rows,
                              int npad, int32_t *scratch, cudaStream_t st);
-cudaError_t launch_init_weights(const uint8_t *y, const WeightLayout &L, const float *w_in,
+// Weights of `faces` faces and the rest non-faces (Table 2), or w_in's, normalised.
+cudaError_t launch_init_weights(const uint8_t *y, int faces, const WeightLayout &L, const float *w_in,
                                 float *w, float *v, RoundState *rs, cudaStream_t st);
 cudaError_t launch_screen(const CUtensorMap *tmap, const float *v, const WeightLayout &L,
                           int lines_per_row, int box_lines, int64_t nfeat, const SearchShape &shape,
