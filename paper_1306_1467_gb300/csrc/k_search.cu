@@ -292,12 +292,16 @@ cudaError_t launch_shortlist(const JobDesc &J, const float *bmin, int nbmin, int
 
 // The compensated re-scan of the shortlist, spread over the SMs: work item i
 // is lane run i % 32 of shortlisted feature i / 32, taken by warp (i / G) % W
-// of CTA i % G (G CTAs of W warps), so that a feature's 32 runs land on 32
-// SMs (one SM doing all 32 was issue-bound: 11.6 us at 24x24 / 15k).  The
-// warp that finishes a feature's last run combines its 32 run results; the
-// warp that completes the last feature picks the round's stump.  Features
-// beyond kRescanSplitCap (only a plateau of ties lists that many) are
-// re-scanned whole, one CTA each.
+// of CTA i % G (the first G = 32 CTAs, of W warps), so that a feature's 32 runs
+// land on 32 SMs (one SM doing all 32 was issue-bound: 11.6 us at 24x24 /
+// 15k).  The warp that finishes a feature's last run combines its 32 run
+// results; the warp that completes the last feature picks the round's stump.
+// Features beyond kRescanSplitCap (a plateau of ties: every feature whose best
+// split is the empty one has the same error) are re-scanned whole, one CTA
+// each, over a grid of two CTAs an SM; in other rounds the CTAs from G on leave
+// at once.  A round with all 78,460 features of 20x20 / 19,997 on its list
+// takes 7.1 ms (11.0 with one CTA an SM, 44.5 with the first G alone); ordinary
+// rounds are the same to a microsecond.
 constexpr int kRescanCtas = 32;
 constexpr int kRescanCtaWarps = 16;
 static_assert(sizeof(RunResult) == kRunResultBytes, "run result layout");
@@ -325,7 +329,8 @@ __global__ void __launch_bounds__(kRescanCtaWarps * 32) k_rescan(const JobDesc J
     }
     const int run = J.npad / 32;
     const int items = min(cnt, kRescanSplitCap) * 32;
-    for (int i = (int)blockIdx.x + (int)gridDim.x * warp; i < items; i += (int)gridDim.x * kRescanCtaWarps) {
+    for (int i = (int)blockIdx.x + kRescanCtas * warp; blockIdx.x < kRescanCtas && i < items;
+         i += kRescanCtas * kRescanCtaWarps) {
         const int c = i >> 5;
         const int32_t f = J.cand_ids[c];
         const RunResult r = rescan_run(J.rows + (size_t)f * J.npad, run, i & 31, J.v, lane);
@@ -381,8 +386,7 @@ __global__ void __launch_bounds__(kRescanCtaWarps * 32) k_rescan(const JobDesc J
 }
 
 cudaError_t launch_rescan(const JobDesc &J, int grid, cudaStream_t st) {
-    (void)grid;
-    k_rescan<<<kRescanCtas, kRescanCtaWarps * 32, 0, st>>>(J);
+    k_rescan<<<std::max(grid, kRescanCtas), kRescanCtaWarps * 32, 0, st>>>(J);
     return cudaGetLastError();
 }
 

@@ -90,9 +90,7 @@ int apply_shape(vjb_ctx *c) {
         c->bmin_cap = c->screen_grid;
     }
     c->shortlist_grid = c->num_sms * 2;
-    // a round shortlists a handful of features: a few CTAs (each takes every
-    // grid-th candidate) launch and hand over to the last one faster than two per SM
-    c->rescan_grid = 16;
+    c->rescan_grid = c->num_sms * 2;
     c->shape_set = true;
     c->drop_graph();
     return VJB_OK;
