@@ -11,7 +11,7 @@
 // entry before the split; s = 0 is always one).  So the feature's least error
 // is min(T+ - max D, T- + min D) over valid splits.
 //
-// Three kernels per search:
+// A search is two steps:
 //  * k_screen (the hot kernel): streams the whole uint16 table once per round
 //    with TMA, gathers v from shared memory, and forms D with FP32 prefix sums.
 //    A warp scans one row: lane k walks its own run of the value order (the
@@ -20,12 +20,11 @@
 //    FP32 warp scan of the 32 run totals per row places every lane's best
 //    prefix in the row.  It writes each feature's FP32 error and each CTA's
 //    minimum.
-//  * k_shortlist: lists every feature whose screened error is within a margin
-//    of the smallest one.
-//  * k_rescan: one CTA per listed feature scans its row again in double-float
-//    (compensated FP32) arithmetic throughout, giving the feature's best split,
-//    polarity and an error to about 1e-14 relative; the last CTA to finish
-//    picks the round's stump: lowest error, then feature, split, +1 before -1.
+//  * the round's tail (k_tail.cu) lists every feature whose screened error is
+//    within a margin of the smallest one and scans the listed rows again in
+//    double-float (compensated FP32) arithmetic throughout, giving each one's
+//    best split, polarity and an error to about 1e-14 relative; the round's
+//    stump is the best of them: lowest error, then feature, split, +1 before -1.
 //
 // Screening error bound (u = 2^-24, sum |v| = T+ + T- = 1 after normalising):
 // a piece's partial sums of at most 24 terms err by at most 24u times the
@@ -236,158 +235,6 @@ int screen_occupancy(const SearchShape &s, int words) {
     else if (s.unroll == 3) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_screen<3>, s.warps * 32, sm);
     else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_screen<2>, s.warps * 32, sm);
     return e == cudaSuccess ? blocks : 0;
-}
-
-// ---- shortlist ------------------------------------------------------------------------
-
-__global__ void __launch_bounds__(256)
-    k_shortlist(const JobDesc J, const float *__restrict__ bmin, int nbmin) {
-    RoundState *rs = J.rs;
-    __shared__ float red[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t b0 = (int64_t)blockIdx.x * blockDim.x + warp * 32;
-    // every load this kernel needs before it can decide, issued together: the
-    // thread's first screened errors, the per-CTA minima and the round state
-    // (one trip to memory instead of three in a row: 4.2 instead of 5.5 us a
-    // launch at 24x24 / 15k under ncu, with the updates' same change)
-    constexpr int kPre = 3;
-    float fe[kPre];
-#pragma unroll
-    for (int q = 0; q < kPre; ++q) {
-        const int64_t f = b0 + q * stride + lane;
-        fe[q] = f < J.nfeat ? J.ferr[f] : INFINITY;
-    }
-    float m = INFINITY;
-    for (int i = threadIdx.x; i < nbmin; i += blockDim.x) m = fminf(m, bmin[i]);
-    if (rs->status != VJB_OK || rs->forced) return;
-    m = warp_min(m);
-    if (lane == 0) red[warp] = m;
-    __syncthreads();
-    m = INFINITY;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fminf(m, red[w]);
-    const float thr = shortlist_threshold(m, rs);
-    if (blockIdx.x == 0 && threadIdx.x == 0) rs->screen_min = m;
-    auto step = [&](int64_t base, float e) {  // base: uniform over the warp
-        const int64_t f = base + lane;
-        const bool take = f < J.nfeat && e <= thr;
-        const uint32_t mask = __ballot_sync(0xffffffffu, take);
-        if (!mask) return;
-        int slot0 = 0;
-        if (lane == 0) slot0 = atomicAdd(&rs->cand_count, __popc(mask));
-        slot0 = __shfl_sync(0xffffffffu, slot0, 0);
-        if (take) J.cand_ids[slot0 + __popc(mask & ((1u << lane) - 1u))] = (int32_t)f;
-    };
-#pragma unroll
-    for (int q = 0; q < kPre; ++q)
-        if (b0 + q * stride < J.nfeat) step(b0 + q * stride, fe[q]);
-    for (int64_t base = b0 + kPre * stride; base < J.nfeat; base += stride)
-        step(base, base + lane < J.nfeat ? J.ferr[base + lane] : INFINITY);
-}
-
-cudaError_t launch_shortlist(const JobDesc &J, const float *bmin, int nbmin, int grid, cudaStream_t st) {
-    k_shortlist<<<grid, 256, 0, st>>>(J, bmin, nbmin);
-    return cudaGetLastError();
-}
-
-// The compensated re-scan of the shortlist, spread over the SMs: work item i
-// is lane run i % 32 of shortlisted feature i / 32, taken by warp (i / G) % W
-// of CTA i % G (the first G = 32 CTAs, of W warps), so that a feature's 32 runs
-// land on 32 SMs (one SM doing all 32 was issue-bound: 11.6 us at 24x24 /
-// 15k).  The warp that finishes a feature's last run combines its 32 run
-// results; the warp that completes the last feature picks the round's stump.
-// Features beyond kRescanSplitCap (a plateau of ties: every feature whose best
-// split is the empty one has the same error) are re-scanned whole, one CTA
-// each, over a grid of two CTAs an SM; in other rounds the CTAs from G on leave
-// at once.  A round with all 78,460 features of 20x20 / 19,997 on its list
-// takes 7.1 ms (11.0 with one CTA an SM, 44.5 with the first G alone); ordinary
-// rounds are the same to a microsecond.
-constexpr int kRescanCtas = 32;
-constexpr int kRescanCtaWarps = 16;
-static_assert(sizeof(RunResult) == kRunResultBytes, "run result layout");
-
-__device__ __forceinline__ RunResult load_run_result(const RunResult *p) {
-    const volatile uint32_t *w = reinterpret_cast<const volatile uint32_t *>(p);
-    RunResult r;
-    r.total.hi = __uint_as_float(w[0]); r.total.lo = __uint_as_float(w[1]);
-    r.mx.hi = __uint_as_float(w[2]);    r.mx.lo = __uint_as_float(w[3]);
-    r.mn.hi = __uint_as_float(w[4]);    r.mn.lo = __uint_as_float(w[5]);
-    r.smx = (int)w[6];                  r.smn = (int)w[7];
-    return r;
-}
-
-__global__ void __launch_bounds__(kRescanCtaWarps * 32) k_rescan(const JobDesc J) {
-    RoundState *rs = J.rs;
-    if (rs->status != VJB_OK || rs->forced) return;
-    __shared__ RunResult rres[32];
-    __shared__ int last_cta;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cnt = rs->cand_count;
-    if (cnt == 0) {  // nothing was listed: stop the job with an error flag
-        if (blockIdx.x == 0 && warp == 0) select_stump_warp(J, 0, lane);
-        return;
-    }
-    const int run = J.npad / 32;
-    const int items = min(cnt, kRescanSplitCap) * 32;
-    for (int i = (int)blockIdx.x + kRescanCtas * warp; blockIdx.x < kRescanCtas && i < items;
-         i += kRescanCtas * kRescanCtaWarps) {
-        const int c = i >> 5;
-        const int32_t f = J.cand_ids[c];
-        const RunResult r = rescan_run(J.rows + (size_t)f * J.npad, run, i & 31, J.v, lane);
-        uint32_t prev = 0;
-        if (lane == 0) {
-            J.runres[i] = r;
-            __threadfence();
-            prev = atomicAdd(&J.cand_runs[c], 1u);
-        }
-        if (__shfl_sync(0xffffffffu, prev, 0) != 31u) continue;
-        // this feature's last run: combine its 32 runs
-        __threadfence();
-        const Candidate cd = combine_runs(J, f, load_run_result(J.runres + c * 32 + lane), lane);
-        if (cnt == 1) {
-            // the only listed feature (most rounds): the stump, picked as the
-            // list would pick it, without the trip through the list
-            if (lane == 0) {
-                J.cand_runs[c] = 0u;
-                Candidate b;
-                b.err_hi = INFINITY; b.err_lo = 0.f; b.feature = INT_MAX; b.split = INT_MAX; b.polarity = 1;
-                b.pad = 0;
-                if (cand_less(cd, b)) b = cd;
-                record_stump(J, 1, b);
-            }
-            continue;
-        }
-        uint32_t done = 0;
-        if (lane == 0) {
-            J.cand_runs[c] = 0u;
-            J.cands[c] = cd;
-            __threadfence();
-            done = atomicAdd(&rs->done_rescan, 1u);
-        }
-        if (__shfl_sync(0xffffffffu, done, 0) == (uint32_t)cnt - 1) {
-            __threadfence();
-            select_stump_warp(J, cnt, lane);
-        }
-    }
-    for (int c = kRescanSplitCap + (int)blockIdx.x; c < cnt; c += (int)gridDim.x) {
-        const Candidate cd = rescan_feature(J, J.cand_ids[c], rres);
-        if (threadIdx.x == 0) {
-            J.cands[c] = cd;
-            __threadfence();
-            last_cta = atomicAdd(&rs->done_rescan, 1u) == (uint32_t)cnt - 1;
-        }
-        __syncthreads();
-        if (last_cta && warp == 0) {
-            __threadfence();
-            select_stump_warp(J, cnt, lane);
-        }
-        __syncthreads();
-    }
-}
-
-cudaError_t launch_rescan(const JobDesc &J, int grid, cudaStream_t st) {
-    k_rescan<<<std::max(grid, kRescanCtas), kRescanCtaWarps * 32, 0, st>>>(J);
-    return cudaGetLastError();
 }
 
 }  // namespace vjb

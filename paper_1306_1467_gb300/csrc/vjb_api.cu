@@ -1,6 +1,6 @@
 // C ABI of the library (declared in include/vjb.h): context ownership,
 // argument checking, the order of the training steps, and the launch sequence
-// of a boosting round (search -> refine -> finalize), replayed as a CUDA graph
+// of a boosting round (search -> tail), replayed as a CUDA graph
 // by vjb_train_strong.
 #include "vjb_host.h"
 
@@ -89,8 +89,6 @@ int apply_shape(vjb_ctx *c) {
         CK(cudaMalloc(&c->d_bmin, sizeof(float) * c->screen_grid));
         c->bmin_cap = c->screen_grid;
     }
-    c->shortlist_grid = c->num_sms * 2;
-    c->rescan_grid = c->num_sms * 2;
     c->shape_set = true;
     c->drop_graph();
     return VJB_OK;
@@ -194,8 +192,6 @@ JobDesc job_desc(const vjb_ctx *c) {
     J.rs = c->d_rs;
     J.ferr = c->d_ferr;
     J.cand_ids = c->d_cand_ids;
-    J.runres = static_cast<RunResult *>(c->d_runres);
-    J.cand_runs = c->d_cand_runs;
     J.cands = c->d_cand;
     J.stumps = c->d_stumps;
     J.diag = c->d_diag;
@@ -215,7 +211,7 @@ int enqueue_update(vjb_ctx *c) {
     return VJB_OK;
 }
 
-// The search kernel of a round, then the rest (shortlist, re-scan, update).
+// The search kernel of a round, then the rest.
 int enqueue_search(vjb_ctx *c) {
     CK(launch_screen(&c->tmap, c->d_v, c->lay, c->lines, c->box_lines, c->nfeat, c->shape,
                      c->screen_grid, c->d_rs, c->d_ferr, c->d_bmin, c->stream));
@@ -223,10 +219,8 @@ int enqueue_search(vjb_ctx *c) {
 }
 
 int enqueue_tail(vjb_ctx *c) {
-    const JobDesc J = job_desc(c);
-    CK(launch_shortlist(J, c->d_bmin, c->screen_grid, c->shortlist_grid, c->stream));
-    CK(launch_rescan(J, c->rescan_grid, c->stream));
-    return enqueue_update(c);
+    CK(launch_tail(job_desc(c), c->d_bmin, c->screen_grid, c->num_sms, c->stream));
+    return VJB_OK;
 }
 
 int enqueue_round(vjb_ctx *c, const EventTriple *ev) {
@@ -414,11 +408,6 @@ int prepare_tables(vjb_ctx *c) {
     if (!c->d_ferr) CK(cudaMalloc(&c->d_ferr, sizeof(float) * c->nfeat));
     if (!c->d_cand) CK(cudaMalloc(&c->d_cand, sizeof(Candidate) * c->nfeat));
     if (!c->d_cand_ids) CK(cudaMalloc(&c->d_cand_ids, sizeof(int32_t) * c->nfeat));
-    if (!c->d_runres) CK(cudaMalloc(&c->d_runres, (size_t)kRunResultBytes * 32 * kRescanSplitCap));
-    if (!c->d_cand_runs) {
-        CK(cudaMalloc(&c->d_cand_runs, sizeof(uint32_t) * kRescanSplitCap));
-        CK(cudaMemset(c->d_cand_runs, 0, sizeof(uint32_t) * kRescanSplitCap));
-    }
     if (!c->d_bmin || !c->tmap_ok) {
         rc = choose_default_shape(c);
         if (rc) return rc;
@@ -459,6 +448,7 @@ int vjb_create(vjb_ctx **out, int device, void *cuda_stream) {
         c->max_smem = (int)prop.sharedMemPerBlockOptin;
     }
     if (e == cudaSuccess) e = set_screen_smem_limit(c->max_smem);
+    if (e == cudaSuccess) e = set_tail_limits();
     if (e == cudaSuccess && cuda_stream) {
         c->stream = static_cast<cudaStream_t>(cuda_stream);
     } else if (e == cudaSuccess) {

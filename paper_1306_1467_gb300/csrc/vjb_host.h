@@ -56,7 +56,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 constexpr int kStageNone = 0, kStageLoaded = 1, kStageIntegral = 2, kStagePrepared = 3;
 constexpr size_t kClassifyPartBytes = 24u << 20;   // windows copied at a time
 constexpr size_t kClassifyKeepBytes = 64u << 20;  // largest workspace kept between calls
-constexpr int kRoundLaunches = 5;  // screen, shortlist, rescan, update a, update b
+constexpr int kRoundLaunches = 3;  // screen, tail, plateau
 
 using EventTriple = std::array<cudaEvent_t, 3>;  // round start, search end, round end
 // A timed round: its events and the one that ends it (its own third event, or
@@ -96,8 +96,6 @@ struct vjb_ctx {
     float *d_ferr = nullptr, *d_bmin = nullptr;
     Candidate *d_cand = nullptr;
     int32_t *d_cand_ids = nullptr;
-    void *d_runres = nullptr;        // re-scan: lane-run results of the split features
-    uint32_t *d_cand_runs = nullptr;  // re-scan: runs done per split feature (kept at zero between rounds)
     uint8_t *d_miss = nullptr;
     int32_t *d_scratch = nullptr;  // table preparation: check state and listed rows
     double *d_partials = nullptr;
@@ -119,7 +117,7 @@ struct vjb_ctx {
     bool tmap_ok = false;
     SearchShape shape{12, 2, 1, 4, 32};
     bool shape_set = false;
-    int screen_grid = 0, shortlist_grid = 0, rescan_grid = 0;
+    int screen_grid = 0;
 
     // graph of one round; with timing on, of its search (graph) and of the
     // rest (graph2), launched with the timing events between them
@@ -147,7 +145,7 @@ struct vjb_ctx {
         dfree(d_rows);
         rows_external = false;
         dfree(d_w); dfree(d_v); dfree(d_wtmp); dfree(d_ferr); dfree(d_bmin); dfree(d_cand);
-        dfree(d_cand_ids); dfree(d_runres); dfree(d_cand_runs); dfree(d_miss); dfree(d_partials); dfree(d_scratch);
+        dfree(d_cand_ids); dfree(d_miss); dfree(d_partials); dfree(d_scratch);
         dfree(d_rs); dfree(d_stumps); dfree(d_last); dfree(d_diag); dfree(d_cls);
         cls_bytes = 0;
         stump_cap = bmin_cap = 0;

@@ -126,12 +126,6 @@ __host__ __device__ __forceinline__ bool entry_flag(uint32_t e, int phys) {
 // compensated.  It is twice a bound on the screening error (see k_search.cu).
 constexpr float kScreenMarginUlps = 72.0f;
 
-// The plain re-scan spreads the first kRescanSplitCap shortlisted features'
-// lane runs over the grid, one run per warp; later ones (a tie plateau) are
-// re-scanned whole by one CTA each.  A run result is 32 bytes.
-constexpr int kRescanSplitCap = 256;
-constexpr int kRunResultBytes = 32;
-
 // Partials of the multi-CTA update kernels (one slot per CTA).
 constexpr int kUpdateThreads = 256;
 constexpr int kUpdateMaxCtas = 4096;
@@ -153,8 +147,6 @@ struct JobDesc {
     float *ferr;
     int32_t *cand_ids;
     struct Candidate *cands;
-    struct RunResult *runres;  // plain re-scan: lane-run results [kRescanSplitCap][32]
-    uint32_t *cand_runs;       // plain re-scan: runs done per candidate [kRescanSplitCap]
     vjb_stump *stumps;
     vjb_round_diag *diag;
     vjb_stump *last;
@@ -232,8 +224,10 @@ cudaError_t launch_init_weights(const uint8_t *y, int faces, const WeightLayout 
 cudaError_t launch_screen(const CUtensorMap *tmap, const float *v, const WeightLayout &L,
                           int lines_per_row, int box_lines, int64_t nfeat, const SearchShape &shape,
                           int grid, RoundState *rs, float *ferr, float *bmin, cudaStream_t st);
-cudaError_t launch_shortlist(const JobDesc &J, const float *bmin, int nbmin, int grid, cudaStream_t st);
-cudaError_t launch_rescan(const JobDesc &J, int grid, cudaStream_t st);
+// What follows a plain round's search (two kernels), on a GPU of `sms` SMs.
+cudaError_t launch_tail(const JobDesc &J, const float *bmin, int nbmin, int sms, cudaStream_t st);
+cudaError_t set_tail_limits();
+// The update alone, with a host-given stump.
 cudaError_t launch_update_a(const JobDesc &J, cudaStream_t st);
 cudaError_t launch_update_b(const JobDesc &J, cudaStream_t st);
 // batched rounds over the jobs of a device job table
