@@ -449,17 +449,21 @@ static cudaError_t launch_sort_ipt(const int32_t *ii_t, int ii_stride, int w, co
 // Then the bank choice of the two weight copies and the run-interleaved write,
 // one 16-byte chunk per thread.
 //
-// What bounds it: shared memory.  16x16 / 15,000 (ncu): shared-memory pipe 66%
-// busy (37 wavefronts per 32 items, half of them the atomics' bank conflicts),
-// issue 49%, ALU 53%, 132 instructions an item.  Ranking with one ballot per
-// digit bit, the form before, was ALU bound at 223 instructions an item.
-// Tables in all, before -> now: 24x24 / 2,003 6.04 -> 2.90 ms, 32x32 / 5,003
-// 31.9 -> 20.0, 24x24 / 15,000 20.9 -> 16.1, 24x24 / 18,300 34.4 -> 26.0.
+// What bounds it: shared memory (16x16 / 15,000 under ncu: its pipe 66% busy, 37
+// wavefronts per 32 items, half of them the atomics' bank conflicts; issue 49%,
+// ALU 53%, 132 instructions an item).  Ranking with one ballot per digit bit,
+// the form before, was ALU bound at 223 instructions an item.  Tables in all,
+// then -> with atomics -> with gaps between the finished runs (kRunGap) and the
+// samples of one copy placed first:
+//   24x24 / 2,003   6.04 ->  2.90 ->  2.54 ms    32x32 / 5,003   31.9 -> 20.0 -> 17.1
+//   24x24 / 10,963  16.4 -> 12.9  -> 12.3         24x24 / 15,000  20.9 -> 16.1 -> 15.7
+//   24x24 / 18,300  34.4 -> 26.0  -> 21.8
 //
 // Threads per CTA grow with the row (128 up to 4,096 samples, 256 up to 8,192,
 // 512 up to 16,384), 1,024 threads an SM in all: small CTAs leave other rows
-// to run while one waits at a barrier.  From 16,385 to 20,480 samples two CTAs of 640 threads still fit
-// an SM (18,300: 26.0 ms, 29.9 with one CTA of 1,024); above, one of 1,024.
+// to run while one waits at a barrier.  From 16,385 to 20,480 samples two CTAs
+// of 640 threads still fit an SM (18,300: 26.0 ms, 29.9 with one CTA of 1,024);
+// above, one of 1,024.
 //
 // Measured and dropped: one pass with a counter per value for spans up to 14
 // bits (one warp ranking a row in order waits its turn behind the other CTA's
@@ -467,6 +471,12 @@ static cudaError_t launch_sort_ipt(const int32_t *ii_t, int ii_stride, int w, co
 // counting or by insertion (28.7 ms); predicated atomics for the last warp's
 // missing items (the compiler wraps each in a branch: 158 instructions).
 constexpr int kPkDigitBits = 8;
+// Words between the 32 lane runs of a finished row in shared memory: runs are a
+// multiple of 8 words long, and without a gap the reads of one place in every
+// run (the write's 16-byte chunks, the refined groups' entries) meet in a few
+// banks, in one when the run is a multiple of 32 (24x24 / 4,096: 4.36 -> 3.65 ms
+// with the gap).
+constexpr int kRunGap = 4;
 constexpr int kPkRadix = 1 << kPkDigitBits;
 
 // Adds to counters in shared memory, as the instructions themselves: the
@@ -493,7 +503,8 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
     extern __shared__ __align__(16) uint8_t smem[];
     uint32_t *skey = reinterpret_cast<uint32_t *>(smem);                        // NP items
     // kPkRadix * WARPS counters, from a multiple of a warp's share of them
-    uint32_t *hist = skey + NP + ((0u - smem_u32(skey + NP)) & (4u * kPkRadix - 1u)) / 4u;
+    uint32_t *hist = skey + NP + 32 * kRunGap;
+    hist += ((0u - smem_u32(hist)) & (4u * kPkRadix - 1u)) / 4u;
     uint32_t *gchoice = hist + kPkRadix * WARPS;                                // GROUPS
     uint32_t *ws = gchoice + GROUPS;                                            // kPkRadix / 32
     int32_t *mm = reinterpret_cast<int32_t *>(ws + kPkRadix / 32);              // 2 * WARPS
@@ -569,14 +580,17 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
     const uint32_t dmask = ((1u << D) - 1u) << 2;  // a digit as a byte offset
     // one stable pass over the D-bit digit from bit `shift` of the values, the
     // items in position order from item(j, p)
-    auto radix_pass = [&](int shift, auto item) {
+    const int run = npad / 32;
+    auto radix_pass = [&](int shift, auto digit, auto item) {
         const int sh = ib + shift - 2;
+        // the last pass leaves the gaps between the runs: position + kRunGap * (position / run)
+        const uint32_t per_run = shift + D >= bits ? 0xffffffffu / (uint32_t)run + 1u : 0u;
         for (int k = lane; k < (1 << D); k += 32) own[k] = 0u;
         __syncwarp();
         auto count = [&](auto whole) {
 #pragma unroll
             for (int j = 0; j < IPT; ++j) {
-                const uint32_t at = ((item(j, pos0 + 32 * j) >> sh) & dmask) | own32;
+                const uint32_t at = (digit(pos0 + 32 * j, sh) & dmask) | own32;
                 shared_add(decltype(whole)::value || j < mine ? at : spare32, 1u);
             }
         };
@@ -623,7 +637,7 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
         // read before any is stored
         uint32_t c[IPT];
 #pragma unroll
-        for (int j = 0; j < IPT; ++j) c[j] = item(j, pos0 + 32 * j);
+        for (int j = 0; j < IPT; ++j) c[j] = item(pos0 + 32 * j);
         __syncthreads();
         // (adds in batches, so that a store does not wait for its own add alone)
         auto place = [&](auto whole) {
@@ -641,7 +655,7 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
 #pragma unroll
                 for (int u = 0; u < BATCH; ++u) {
                     const int j = j0 + u;
-                    if (j < IPT && (decltype(whole)::value || j < mine)) skey[to[u]] = c[j];
+                    if (j < IPT && (decltype(whole)::value || j < mine)) skey[to[u] + kRunGap * __umulhi(to[u], per_run)] = c[j];
                 }
             }
         };
@@ -651,13 +665,19 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
     };
     // (a row of one value takes a pass too: every digit 0, the items in order)
     if (narrow)
-        radix_pass(0, [&](int j, int p) { return (((uint32_t)val16[p] - (uint32_t)lo) << ib) + (uint32_t)p; });
+        radix_pass(
+            0, [&](int p, int) { return ((uint32_t)val16[p] - (uint32_t)lo) << 2; },
+            [&](int p) { return (((uint32_t)val16[p] - (uint32_t)lo) << ib) + (uint32_t)p; });
     else
-        radix_pass(0, [&](int j, int p) { return ((skey[p] - (uint32_t)lo) << ib) + (uint32_t)p; });
-    for (int shift = D; shift < bits; shift += D) radix_pass(shift, [&](int j, int p) { return skey[p]; });
+        radix_pass(
+            0, [&](int p, int) { return (skey[p] - (uint32_t)lo) << 2; },
+            [&](int p) { return ((skey[p] - (uint32_t)lo) << ib) + (uint32_t)p; });
+    for (int shift = D; shift < bits; shift += D) 
+        radix_pass(
+            shift, [&](int p, int sh) { return skey[p] >> sh; }, [&](int p) { return skey[p]; });
 
     uint16_t *out = rows + (size_t)blockIdx.x * npad;
-    const int run = npad / 32;
+    const int pitch = run + kRunGap;  // from run to run in skey
     if (L.dual) {
         // bank-balanced copy choice per gather group (see k_sort_rows): each
         // entry goes to the less loaded of its two banks, one thread a group.
@@ -666,7 +686,6 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
         // counter space) and taken by a warp each, a lane per entry: while an
         // entry of such a bank has its other bank below 2, the first of them
         // moves there.
-        const bool part = L.nb < n;  // samples from nb on have one copy only
         uint32_t *rlist = hist;      // (group, masks) of the groups to refine
         auto bank_bits = [&](uint32_t x, uint32_t &a, uint32_t &b) {  // x: a word of skey (its bits 0-9 are the index's)
             a = __funnelshift_l(0u, 1u, x);                    // 1 << (i mod 32)
@@ -674,75 +693,100 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
         };
         if (threadIdx.x == 0) mm[0] = 0;
         __syncthreads();
-        for (int g = threadIdx.x; g < run; g += TH) {
-            uint32_t m1 = 0u, m2 = 0u, m3 = 0u, mask = 0u;
-            const int kend = min(32, (n - g + run - 1) / run);  // entries k * run + g < n
-            auto entry = [&](int k) {
-                const uint32_t x = skey[k * run + g];
-                uint32_t a, b;
-                bank_bits(x, a, b);
-                if (part && (int)(x & imask) >= L.nb) b = a;
-                // bank b is less loaded if it has no entry and a has one, or
-                // has one and a has two; without branches
-                uint32_t to;
-                asm("{\n\t.reg .pred p, q;\n\t.reg .b32 t;\n\t"
-                    "and.b32 t, %2, %4;\n\tsetp.ne.u32 p, t, 0;\n\t"
-                    "and.b32 t, %2, %5;\n\tsetp.eq.and.u32 p, t, 0, p;\n\t"
-                    "and.b32 t, %3, %4;\n\tsetp.ne.u32 q, t, 0;\n\t"
-                    "and.b32 t, %3, %5;\n\tsetp.eq.and.u32 q, t, 0, q;\n\t"
-                    "or.pred p, p, q;\n\t"
-                    "selp.b32 %0, %5, %4, p;\n\t"
-                    "@p or.b32 %1, %1, %6;\n\t}"
-                    : "=r"(to), "+r"(mask)
-                    : "r"(m1), "r"(m2), "r"(a), "r"(b), "r"(1u << k));
-                m3 |= m2 & to;
-                m2 |= m1 & to;
-                m1 |= to;
-            };
-            if (kend == 32) {
+        auto choose = [&](auto partial) {
+            for (int g = threadIdx.x; g < run; g += TH) {
+                uint32_t m1 = 0u, m2 = 0u, m3 = 0u, mask = 0u;
+                const int kend = min(32, (n - g + run - 1) / run);  // entries k * run + g < n
+                const uint32_t *first = skey + g;
+                auto put = [&](uint32_t to) {
+                    m3 |= m2 & to;
+                    m2 |= m1 & to;
+                    m1 |= to;
+                };
+                auto entry = [&](int k) {
+                    const uint32_t x = first[k * pitch];
+                    uint32_t a, b;
+                    bank_bits(x, a, b);
+                    if (decltype(partial)::value && (int)(x & imask) >= L.nb) a = b = 0u;  // placed before
+                    // bank b is less loaded if it has no entry and a has one,
+                    // or has one and a has two; without branches
+                    uint32_t to;
+                    asm("{\n\t.reg .pred p, q;\n\t.reg .b32 t;\n\t"
+                        "and.b32 t, %2, %4;\n\tsetp.ne.u32 p, t, 0;\n\t"
+                        "and.b32 t, %2, %5;\n\tsetp.eq.and.u32 p, t, 0, p;\n\t"
+                        "and.b32 t, %3, %4;\n\tsetp.ne.u32 q, t, 0;\n\t"
+                        "and.b32 t, %3, %5;\n\tsetp.eq.and.u32 q, t, 0, q;\n\t"
+                        "or.pred p, p, q;\n\t"
+                        "selp.b32 %0, %5, %4, p;\n\t"
+                        "@p or.b32 %1, %1, %6;\n\t}"
+                        : "=r"(to), "+r"(mask)
+                        : "r"(m1), "r"(m2), "r"(a), "r"(b), "r"(1u << k));
+                    put(to);
+                };
+                if (decltype(partial)::value) {
+                    // the samples with one copy first: those with two fill the gaps
 #pragma unroll 8
-                for (int k = 0; k < 32; ++k) entry(k);
-            } else {
-                for (int k = 0; k < kend; ++k) entry(k);
-                const uint32_t to = 1u << (n & 31);  // the padding word, read as a broadcast
-                m3 |= m2 & to;
-                m2 |= m1 & to;
-                m1 |= to;
+                    for (int k = 0; k < kend; ++k) {
+                        const uint32_t x = first[k * pitch];
+                        put((int)(x & imask) >= L.nb ? __funnelshift_l(0u, 1u, x) : 0u);
+                    }
+                }
+                if (kend == 32) {
+#pragma unroll 8
+                    for (int k = 0; k < 32; ++k) entry(k);
+                } else {
+                    for (int k = 0; k < kend; ++k) entry(k);
+                    put(1u << (n & 31));  // the padding word, read as a broadcast
+                }
+                gchoice[g] = mask;
+                // (rows above 20,480 samples: so few entries have two copies that
+                // refining buys no search time; 24,000: 5 us for 2.9 ms)
+                if (m3 && (TH < 1024 || !decltype(partial)::value)) {
+                    const int q = atomicAdd(&mm[0], 1);
+                    reinterpret_cast<uint4 *>(rlist)[q] = make_uint4((uint32_t)g, m1, m2, m3);
+                }
             }
-            gchoice[g] = mask;
-            if (m3) {
-                const int q = atomicAdd(&mm[0], 1);
-                rlist[4 * q] = (uint32_t)g;
-                rlist[4 * q + 1] = m1;
-                rlist[4 * q + 2] = m2;
-                rlist[4 * q + 3] = m3;
-            }
-        }
+        };
+        if (L.nb < n) choose(std::true_type{});  // samples from nb on have one copy only
+        else choose(std::false_type{});
         __syncthreads();
         const int nref = mm[0];
+        // (the next group's words are on their way while this one is taken)
+        struct Group {
+            int g;
+            uint32_t m1, m2, m3, mask, x;
+        } cur, next;
+        auto fetch = [&](int q, Group &k) {
+            if (q >= nref) return;
+            const uint4 l = reinterpret_cast<const uint4 *>(rlist)[q];
+            k.g = (int)l.x;
+            k.m1 = l.y;
+            k.m2 = l.z;
+            k.m3 = l.w;
+            k.mask = gchoice[k.g];
+            k.x = skey[lane * pitch + k.g];
+        };
+        fetch(wp, next);
         for (int q = wp; q < nref; q += WARPS) {
-            const int g = (int)rlist[4 * q];
-            uint32_t m1 = rlist[4 * q + 1], m2 = rlist[4 * q + 2], m3 = rlist[4 * q + 3];
-            uint32_t mask = gchoice[g];
-            const bool in = lane * run + g < n;
-            const uint32_t x = in ? skey[lane * run + g] : 0u;
+            cur = next;
+            fetch(q + WARPS, next);
             uint32_t a, b;
-            bank_bits(x, a, b);
-            bool onb = (mask >> lane) & 1u;
-            const bool can = in && (int)(x & imask) < L.nb;
+            bank_bits(cur.x, a, b);
+            bool onb = (cur.mask >> lane) & 1u;
+            const bool can = lane * run + cur.g < n && (int)(cur.x & imask) < L.nb;
             for (;;) {
-                const uint32_t cur = onb ? b : a, oth = onb ? a : b;
-                const uint32_t moves = __ballot_sync(0xffffffffu, can && (m3 & cur) && !(m2 & oth));
+                const uint32_t now = onb ? b : a, oth = onb ? a : b;
+                const uint32_t moves = __ballot_sync(0xffffffffu, can && (cur.m3 & now) && !(cur.m2 & oth));
                 if (!moves) break;
                 const int first = __ffs(moves) - 1;
-                const uint32_t from = __shfl_sync(0xffffffffu, cur, first), to = __shfl_sync(0xffffffffu, oth, first);
-                m3 &= ~from;
-                m2 |= m1 & to;
-                m1 |= to;
-                mask ^= 1u << first;
+                const uint32_t from = __shfl_sync(0xffffffffu, now, first), to = __shfl_sync(0xffffffffu, oth, first);
+                cur.m3 &= ~from;
+                cur.m2 |= cur.m1 & to;
+                cur.m1 |= to;
+                cur.mask ^= 1u << first;
                 if (lane == first) onb = !onb;
             }
-            if (lane == 0) gchoice[g] = mask;
+            if (lane == 0) gchoice[cur.g] = cur.mask;
         }
         __syncthreads();
     }
@@ -754,11 +798,13 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
         const int k = c & 31, t = c >> 5;
         const int p0 = k * run + t * kChunkElems;
         uint32_t cp[kChunkElems + 1];
-        const uint4 lo4 = *reinterpret_cast<const uint4 *>(skey + p0);
-        const uint4 hi4 = *reinterpret_cast<const uint4 *>(skey + p0 + 4);
+        const uint32_t *at = skey + k * pitch + t * kChunkElems;
+        const uint4 lo4 = *reinterpret_cast<const uint4 *>(at);
+        const uint4 hi4 = *reinterpret_cast<const uint4 *>(at + 4);
         cp[0] = lo4.x; cp[1] = lo4.y; cp[2] = lo4.z; cp[3] = lo4.w;
         cp[4] = hi4.x; cp[5] = hi4.y; cp[6] = hi4.z; cp[7] = hi4.w;
-        cp[8] = p0 + kChunkElems < n ? skey[p0 + kChunkElems] : 0u;
+        // (the run's last chunk is followed by the next run, past the gap)
+        cp[8] = p0 + kChunkElems < n ? at[kChunkElems + (t == run / kChunkElems - 1 ? kRunGap : 0)] : 0u;
         uint32_t gc[kChunkElems] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
         if (L.dual) {
             const uint4 g0 = *reinterpret_cast<const uint4 *>(gchoice + t * kChunkElems);
@@ -810,7 +856,7 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
 
 template <int IPT, int TH>
 static size_t sort_packed_smem() {
-    return (size_t)(TH * IPT + kPkRadix + kPkRadix * (TH / 32) + TH * IPT / 32 + kPkRadix / 32 + 2 * (TH / 32) + 32) * 4;
+    return (size_t)(TH * IPT + 32 * kRunGap + kPkRadix + kPkRadix * (TH / 32) + TH * IPT / 32 + kPkRadix / 32 + 2 * (TH / 32) + 32) * 4;
 }
 
 template <int IPT, int TH>
@@ -865,14 +911,18 @@ cudaError_t launch_sort_rows(const int32_t *ii_t, const uint16_t *ii16, int ii_s
     else
     VJB_PK_CASE(8, 128)
     VJB_PK_CASE(16, 128)
+    VJB_PK_CASE(20, 128)
     VJB_PK_CASE(24, 128)
+    VJB_PK_CASE(28, 128)
     VJB_PK_CASE(32, 128)
     VJB_PK_CASE(20, 256)
     VJB_PK_CASE(24, 256)
     VJB_PK_CASE(28, 256)
     VJB_PK_CASE(32, 256)
     VJB_PK_CASE(20, 512)
+    VJB_PK_CASE(22, 512)
     VJB_PK_CASE(24, 512)
+    VJB_PK_CASE(26, 512)
     VJB_PK_CASE(28, 512)
     VJB_PK_CASE(30, 512)
     VJB_PK_CASE(32, 512)
