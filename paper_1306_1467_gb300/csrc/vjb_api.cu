@@ -33,16 +33,31 @@ int32_t *flags_ptr(vjb_ctx *c) {
     return reinterpret_cast<int32_t *>(reinterpret_cast<char *>(c->d_rs) + offsetof(RoundState, flags));
 }
 
-// Canonical enumeration (types 3H, 3V, 2H, 2V, 4; then width, height, y, x).
+// Feature k of the canonical list (haar_count).
+vjb_feature feature_at(int W, int H, int64_t k) {
+    int t = 0;
+    for (; k >= haar_count(t, W, H); ++t) k -= haar_count(t, W, H);
+    const HaarBase b = haar_base(t);
+    const int64_t heights = haar_places(H, b.h, H / b.h);
+    int fw = b.w, fh = b.h;
+    for (; k >= (W - fw + 1) * heights; fw += b.w) k -= (W - fw + 1) * heights;
+    const int64_t nx = W - fw + 1;
+    for (; k >= nx * (H - fh + 1); fh += b.h) k -= nx * (H - fh + 1);
+    return vjb_feature{(uint8_t)t, (uint8_t)(k % nx), (uint8_t)(k / nx), (uint8_t)fw, (uint8_t)fh};
+}
+
+// The whole list, for a caller who asks for it.
 void enumerate_host(int W, int H, std::vector<vjb_feature> &out) {
-    static const int bw[5] = {3, 1, 2, 1, 2}, bh[5] = {1, 3, 1, 2, 2};
-    out.clear();
-    for (int t = 0; t < 5; ++t)
-        for (int fw = bw[t]; fw <= W; fw += bw[t])
-            for (int fh = bh[t]; fh <= H; fh += bh[t])
+    out.resize((size_t)haar_count(W, H));
+    vjb_feature *f = out.data();
+    for (int t = 0; t < 5; ++t) {
+        const HaarBase b = haar_base(t);
+        for (int fw = b.w; fw <= W; fw += b.w)
+            for (int fh = b.h; fh <= H; fh += b.h)
                 for (int y = 0; y + fh <= H; ++y)
                     for (int x = 0; x + fw <= W; ++x)
-                        out.push_back(vjb_feature{(uint8_t)t, (uint8_t)x, (uint8_t)y, (uint8_t)fw, (uint8_t)fh});
+                        *f++ = vjb_feature{(uint8_t)t, (uint8_t)x, (uint8_t)y, (uint8_t)fw, (uint8_t)fh};
+    }
 }
 
 int make_tensor_map(vjb_ctx *c) {
@@ -357,21 +372,22 @@ int copy_stump_out(vjb_ctx *c, vjb_stump *out) {
 // Feature values (K2) and sort (K3) a tile of features at a time, then a check
 // of the finished table.
 int prepare_tables(vjb_ctx *c) {
-    if (c->feats.empty()) {
-        enumerate_host(c->w, c->h, c->feats);
-        c->nfeat = (int64_t)c->feats.size();
+    if (!c->d_feat) {
+        c->nfeat = haar_count(c->w, c->h);
         if (c->nfeat == 0 || c->nfeat > 0x7fffffffLL)
             return fail(VJB_EINVAL, "window %dx%d has %lld features", c->w, c->h, (long long)c->nfeat);
-        std::vector<DevFeature> df((size_t)c->nfeat);
-        for (size_t k = 0; k < df.size(); ++k) {
-            const vjb_feature &f = c->feats[k];
-            df[k] = DevFeature{f.type, f.x, f.y, f.w, f.h, 0, 0, 0};
-        }
-        CK(cudaMalloc(&c->d_feat, sizeof(DevFeature) * df.size()));
-        CK(cudaMemcpy(c->d_feat, df.data(), sizeof(DevFeature) * df.size(), cudaMemcpyHostToDevice));
         c->npad = (c->n + kRowAlign - 1) / kRowAlign * kRowAlign;
         c->lines = c->npad / kLineElems;
         c->box_lines = 0;  // set with the search shape
+        DevFeature *feat = nullptr;
+        CK(cudaMalloc(&feat, sizeof(DevFeature) * (size_t)c->nfeat));
+        const cudaError_t ef = launch_enumerate(c->w, c->h, feat, c->stream);
+        if (ef != cudaSuccess) {
+            cudaFree(feat);
+            return fail(VJB_ECUDA, "feature list: %s", cudaGetErrorString(ef));
+        }
+        c->d_feat = feat;
+        c->launches += 1;
     }
     if (!c->d_rows) {
         if (c->rows_external) return fail(VJB_ESTATE, "external table not set");
@@ -520,7 +536,10 @@ int vjb_enumerate_haar(vjb_ctx *c, int64_t *count, vjb_feature *out) {
         c->stage = kStagePrepared;
     }
     *count = c->nfeat;
-    if (out) memcpy(out, c->feats.data(), sizeof(vjb_feature) * c->feats.size());
+    if (out) {
+        if (c->feats.empty()) enumerate_host(c->w, c->h, c->feats);
+        memcpy(out, c->feats.data(), sizeof(vjb_feature) * c->feats.size());
+    }
     return VJB_OK;
 }
 
@@ -710,7 +729,7 @@ int vjb_classify(vjb_ctx *c, const uint8_t *pixels, int32_t n, const vjb_stump *
         if (s.feature < 0 || s.feature >= c->nfeat || (s.polarity != 1 && s.polarity != -1) || std::isnan(s.alpha))
             return fail(VJB_EINVAL, "stump %d is not a stump of this window size", t);
         half += s.alpha;
-        const vjb_feature &f = c->feats[(size_t)s.feature];
+        const vjb_feature f = feature_at(c->w, c->h, s.feature);
         cs[(size_t)t] = ClassStump{DevFeature{f.type, f.x, f.y, f.w, f.h, 0, 0, 0}, s.threshold, s.polarity, s.alpha};
     }
     half *= 0.5;  // C(x) = 1 iff sum alpha_t h_t(x) >= 1/2 sum alpha_t

@@ -89,10 +89,8 @@ int batch_encode_maps(vjb_batch *b) {
 }
 
 int64_t table_lines(int n, int h, int w) {
-    std::vector<vjb_feature> f;
-    enumerate_host(w, h, f);
     const int64_t npad = (n + kRowAlign - 1) / kRowAlign * kRowAlign;
-    return (int64_t)f.size() * (npad / kLineElems);
+    return haar_count(w, h) * (npad / kLineElems);
 }
 
 bool arena_take(vjb_batch *b, int64_t count, int64_t *first) {

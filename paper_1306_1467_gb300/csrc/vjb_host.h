@@ -112,7 +112,7 @@ struct vjb_ctx {
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t cls_ev[4] = {nullptr, nullptr, nullptr, nullptr};
 
-    std::vector<vjb_feature> feats;
+    std::vector<vjb_feature> feats;  // the feature list, once a caller has asked for it
     CUtensorMap tmap;
     bool tmap_ok = false;
     SearchShape shape{12, 2, 1, 4, 32};
@@ -171,7 +171,6 @@ struct vjb_ctx {
 namespace vjb {
 
 // Context helpers (vjb_api.cu) that the batch and serving code reuse.
-void enumerate_host(int w, int h, std::vector<vjb_feature> &out);
 int ensure_stump_cap(vjb_ctx *c, int need);
 JobDesc job_desc(const vjb_ctx *c);
 int validate_labels(const uint8_t *y, int n);

@@ -15,6 +15,30 @@ struct DevFeature {
     uint8_t type, x, y, w, h, pad0, pad1, pad2;
 };
 
+// The canonical feature list of a W x H window (types 3H, 3V, 2H, 2V, 4; inside
+// a type by width, height, y, x ascending).  Type t's features have widths and
+// heights that are multiples of its base size.
+struct HaarBase {
+    int w, h;
+};
+__host__ __device__ __forceinline__ HaarBase haar_base(int t) {
+    return HaarBase{t == VJB_HAAR_3H ? 3 : (t == VJB_HAAR_3V || t == VJB_HAAR_2V ? 1 : 2),
+                    t == VJB_HAAR_3V ? 3 : (t == VJB_HAAR_3H || t == VJB_HAAR_2H ? 1 : 2)};
+}
+// Positions of boxes b, 2b, ..., m b long on a line of E.
+__host__ __device__ __forceinline__ int64_t haar_places(int E, int b, int m) {
+    return (int64_t)m * (E + 1) - (int64_t)b * m * (m + 1) / 2;
+}
+__host__ __device__ __forceinline__ int64_t haar_count(int t, int W, int H) {
+    const HaarBase b = haar_base(t);
+    return haar_places(W, b.w, W / b.w) * haar_places(H, b.h, H / b.h);
+}
+__host__ __device__ __forceinline__ int64_t haar_count(int W, int H) {
+    int64_t c = 0;
+    for (int t = 0; t < 5; ++t) c += haar_count(t, W, H);
+    return c;
+}
+
 // Where the signed weights v_i (+w_i for a face, -w_i for a non-face) live.
 // Table entries are word offsets into this array.  With two copies, copy A
 // holds v_i at word i and copy B at word off_b + rot(i), where rot rotates
@@ -212,6 +236,8 @@ cudaError_t launch_strong_classify(const int32_t *ii_t, int ii_stride, int n, in
 bool classify_fits(int h, int w, int max_smem);
 cudaError_t launch_classify_windows(const uint8_t *px, int n, int h, int w, const ClassStump *stumps, int T,
                                     double half_alpha, uint8_t *labels, double *scores, cudaStream_t st);
+// The feature list of a w x h window.
+cudaError_t launch_enumerate(int w, int h, DevFeature *feat, cudaStream_t st);
 cudaError_t launch_feature_values(const int32_t *ii_t, int ii_stride, int n, int w,
                                   const DevFeature *feat, int64_t f0, int64_t nf, int32_t *out,
                                   cudaStream_t st);
