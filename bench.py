@@ -587,7 +587,7 @@ def batch_comparison(a, device: int = 0) -> dict:
                         "shape": {**{k: info[k] for k in ("warps", "stages", "unroll", "box_lines")},
                                   "schedule": {-1: "partitioned", -2: "interleaved"}.get(
                                       info["rows_per_warp"], f"work queue, {info['rows_per_warp']} rows per warp and item")},
-                        "setup_s": setup_s, "launches_per_round": 6},
+                        "setup_s": setup_s, "launches_per_round": 7},
             "roofline": {"kernel": "k_bscreen", "bound": "hbm", "achieved": search_gbs, "peak": peak,
                          "peak_source": f"{peak_src} hbm_gbs", "unit": "GB/s", "frac": search_gbs / peak,
                          "algorithmic_bytes_per_launch": round_bytes, "avg_launch_ms": search_ms,

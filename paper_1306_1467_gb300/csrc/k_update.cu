@@ -178,6 +178,21 @@ cudaError_t launch_bupdate_a(const JobDesc *jobs, BatchMeta *meta, int grid, cud
     return cudaGetLastError();
 }
 
+// End of a batched round: its outcome for the host.
+__global__ void k_bend(const JobDesc *__restrict__ jobs, const BatchMeta *__restrict__ meta, BatchSeen *seen) {
+    const int j = threadIdx.x;
+    if (j == 0) seen->flags = meta->flags;
+    if (j < meta->njobs) {
+        const RoundState *rs = jobs[j].rs;
+        seen->job[j] = JobSeen{rs->status, rs->rounds, rs->flags, 0};
+    }
+}
+
+cudaError_t launch_bend(const JobDesc *jobs, const BatchMeta *meta, BatchSeen *seen, cudaStream_t st) {
+    k_bend<<<1, kMaxBatchJobs, 0, st>>>(jobs, meta, seen);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_bupdate_b(const JobDesc *jobs, BatchMeta *meta, int grid, cudaStream_t st) {
     k_bupdate<false><<<grid, kUpdateThreads, 0, st>>>(jobs, meta);
     return cudaGetLastError();

@@ -288,8 +288,19 @@ int ensure_graph(vjb_ctx *c) {
 }
 
 int read_state(vjb_ctx *c, RoundState *rs) {
-    CK(cudaMemcpyAsync(rs, c->d_rs, sizeof(RoundState), cudaMemcpyDeviceToHost, c->stream));
+    c->seen_now = false;
+    CK(cudaMemcpyAsync(&c->seen, c->d_rs, sizeof(RoundRecord), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    c->seen_now = true;
+    *rs = c->seen.rs;
+    return VJB_OK;
+}
+
+// The state at the start of a call that trains: every such call reads it at its
+// end, so it is read again only after a load or new weights (a read costs 10 us).
+int known_state(vjb_ctx *c, RoundState *rs) {
+    if (!c->seen_now) return read_state(c, rs);
+    *rs = c->seen.rs;
     return VJB_OK;
 }
 
@@ -344,8 +355,8 @@ int load_common(vjb_ctx *c, const uint8_t *pixels, const uint8_t *labels, int32_
         CK(cudaMemset(c->d_v, 0, sizeof(float) * c->lay.words));
         CK(cudaMalloc(&c->d_miss, (size_t)n));
         CK(cudaMalloc(&c->d_partials, sizeof(double) * 3 * kUpdateMaxCtas));
-        CK(cudaMalloc(&c->d_rs, sizeof(RoundState)));
-        CK(cudaMalloc(&c->d_last, sizeof(vjb_stump)));
+        CK(cudaMalloc(&c->d_rs, sizeof(RoundRecord)));
+        c->d_last = reinterpret_cast<vjb_stump *>(reinterpret_cast<char *>(c->d_rs) + offsetof(RoundRecord, last));
         rc = ensure_stump_cap(c, 1024);
         if (rc) return rc;
     }
@@ -353,8 +364,8 @@ int load_common(vjb_ctx *c, const uint8_t *pixels, const uint8_t *labels, int32_
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     CK(cudaMemcpyAsync(c->d_px, pixels, (size_t)n * h * w, kind, c->stream));
     CK(cudaMemcpyAsync(c->d_y, hy.data(), (size_t)n, cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemsetAsync(c->d_rs, 0, sizeof(RoundState), c->stream));
-    CK(cudaMemsetAsync(c->d_last, 0, sizeof(vjb_stump), c->stream));
+    c->seen_now = false;
+    CK(cudaMemsetAsync(c->d_rs, 0, sizeof(RoundRecord), c->stream));
     CK(launch_init_weights(c->d_y, faces, c->lay, nullptr, c->d_w, c->d_v, c->d_rs, c->stream));
     c->launches += 1;
     CK(cudaStreamSynchronize(c->stream));
@@ -362,11 +373,9 @@ int load_common(vjb_ctx *c, const uint8_t *pixels, const uint8_t *labels, int32_
     return VJB_OK;
 }
 
-int copy_stump_out(vjb_ctx *c, vjb_stump *out) {
-    if (!out) return VJB_OK;
-    CK(cudaMemcpyAsync(out, c->d_last, sizeof(vjb_stump), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    return VJB_OK;
+// The last stump, as read with the state at the end of a call.
+void copy_stump_out(const vjb_ctx *c, vjb_stump *out) {
+    if (out) *out = c->seen.last;
 }
 
 // Feature values (K2) and sort (K3) a tile of features at a time, then a check
@@ -550,9 +559,10 @@ int vjb_train_round(vjb_ctx *c, vjb_stump *out) {
     int rc = set_dev(c);
     if (rc) return rc;
     RoundState rs;
-    rc = read_state(c, &rs);
+    rc = known_state(c, &rs);
     if (rc) return rc;
     if (rs.status == VJB_OK) {
+        c->seen_now = false;
         rc = ensure_stump_cap(c, rs.rounds + 1);
         if (rc) return rc;
         EventTriple ev{};
@@ -568,8 +578,7 @@ int vjb_train_round(vjb_ctx *c, vjb_stump *out) {
         if (rc) return rc;
     }
     if (rs.flags) return device_flags_error(rs);
-    rc = copy_stump_out(c, out);
-    if (rc) return rc;
+    copy_stump_out(c, out);
     return rs.status;
 }
 
@@ -581,10 +590,11 @@ int vjb_train_strong(vjb_ctx *c, int32_t T, vjb_stump *out, int32_t *rounds_done
     int rc = set_dev(c);
     if (rc) return rc;
     RoundState rs;
-    rc = read_state(c, &rs);
+    rc = known_state(c, &rs);
     if (rc) return rc;
     const int r0 = rs.rounds;
     if (rs.status == VJB_OK && T > 0) {
+        c->seen_now = false;
         rc = ensure_stump_cap(c, r0 + T);
         if (rc) return rc;
         rc = ensure_graph(c);
@@ -644,6 +654,7 @@ int vjb_set_weights(vjb_ctx *c, const float *wts) {
     if (!(s > 0.0)) return fail(VJB_EINVAL, "weights sum to zero");
     int rc = set_dev(c);
     if (rc) return rc;
+    c->seen_now = false;
     CK(cudaMemcpyAsync(c->d_wtmp, wts, sizeof(float) * c->n, cudaMemcpyHostToDevice, c->stream));
     CK(launch_init_weights(c->d_y, 0, c->lay, c->d_wtmp, c->d_w, c->d_v, c->d_rs, c->stream));
     c->launches += 1;
@@ -660,9 +671,10 @@ int vjb_force_stump(vjb_ctx *c, int32_t feature, int32_t threshold, int32_t pola
     int rc = set_dev(c);
     if (rc) return rc;
     RoundState rs;
-    rc = read_state(c, &rs);
+    rc = known_state(c, &rs);
     if (rc) return rc;
     if (rs.status == VJB_OK) {
+        c->seen_now = false;
         rc = ensure_stump_cap(c, rs.rounds + 1);
         if (rc) return rc;
         int32_t f4[4] = {1, feature, threshold, polarity};
@@ -675,8 +687,7 @@ int vjb_force_stump(vjb_ctx *c, int32_t feature, int32_t threshold, int32_t pola
         if (rc) return rc;
     }
     if (rs.flags) return device_flags_error(rs);
-    rc = copy_stump_out(c, out);
-    if (rc) return rc;
+    copy_stump_out(c, out);
     return rs.status;
 }
 

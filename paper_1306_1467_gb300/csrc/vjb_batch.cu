@@ -17,6 +17,7 @@ struct BatchSlot {
     int32_t id = -1;
     int64_t line_base = 0, line_count = 0;
     int32_t round_target = 0;
+    JobSeen seen{VJB_OK, 0, 0, 0};  // as of the last batched round it was part of
 };
 
 constexpr int kBatchMaxWords = 32768;  // weights of any job fit the search kernel's shared memory
@@ -36,6 +37,8 @@ struct vjb_batch {
     int32_t next_id = 0;
     JobDesc *d_jobs = nullptr;
     BatchMeta *d_meta = nullptr;
+    BatchSeen *seen = nullptr;  // mapped host memory, written at the end of every round
+    int32_t flags = 0;          // error flags of the rounds so far
     WorkItem *d_items = nullptr;
     int items_cap = 0;
     bool dirty = true;  // the device job table must be rebuilt
@@ -183,6 +186,7 @@ int batch_enqueue_round(vjb_batch *b, int part) {
         CK(launch_brescan(b->d_jobs, b->d_meta, std::min(g, 128), b->stream));
         CK(launch_bupdate_a(b->d_jobs, b->d_meta, g * 4, b->stream));
         CK(launch_bupdate_b(b->d_jobs, b->d_meta, g * 4, b->stream));
+        CK(launch_bend(b->d_jobs, b->d_meta, b->seen, b->stream));
     }
     return VJB_OK;
 }
@@ -257,14 +261,12 @@ bool batch_shape_ok(const vjb_batch *b, const SearchShape &s) {
 
 // Largest number of rounds a job of the batch still wants (0 when all are
 // done); grows the jobs' stump records to their targets.
-int batch_rounds_wanted(vjb_batch *b, int *want, std::vector<RoundState> *states = nullptr) {
+int batch_rounds_wanted(vjb_batch *b, int *want, std::vector<JobSeen> *states = nullptr) {
     *want = 0;
-    std::vector<RoundState> st(b->slots.size());
-    for (size_t k = 0; k < st.size(); ++k)
-        CK(cudaMemcpyAsync(&st[k], b->slots[k].ctx->d_rs, sizeof(RoundState), cudaMemcpyDeviceToHost, b->stream));
-    CK(cudaStreamSynchronize(b->stream));
+    std::vector<JobSeen> st(b->slots.size());
     for (size_t k = 0; k < st.size(); ++k) {
         BatchSlot &s = b->slots[k];
+        st[k] = s.seen;
         if (st[k].status == VJB_OK && !st[k].flags) *want = std::max(*want, s.round_target - st[k].rounds);
         if (s.round_target > s.ctx->stump_cap) {
             const int rc = ensure_stump_cap(s.ctx, s.round_target);
@@ -303,7 +305,7 @@ int batch_run(vjb_batch *b, int R, float *ms) {
             } else {
                 CK(cudaGraphLaunch(b->gexec, b->stream));
             }
-            b->launches += 6;
+            b->launches += 7;
         }
         if (ms) {
             CK(cudaEventRecord(e1, b->stream));
@@ -316,9 +318,12 @@ int batch_run(vjb_batch *b, int R, float *ms) {
         *ms = 0.f;
     }
     CK(cudaStreamSynchronize(b->stream));
-    BatchMeta m;
-    CK(cudaMemcpy(&m, b->d_meta, sizeof m, cudaMemcpyDeviceToHost));
-    if (m.flags) return fail(VJB_EDEVICE, "batched kernel error flags 0x%x", m.flags);
+    if (R > 0 && !b->slots.empty()) {
+        // (the slots are the job table's rows: nothing has changed them since batch_sync)
+        b->flags = b->seen->flags;
+        for (size_t k = 0; k < b->slots.size(); ++k) b->slots[k].seen = b->seen->job[k];
+    }
+    if (b->flags) return fail(VJB_EDEVICE, "batched kernel error flags 0x%x", b->flags);
     return VJB_OK;
 }
 
@@ -341,6 +346,7 @@ int vjb_batch_create(vjb_batch **out, int device, void *cuda_stream, int64_t tab
         if (b->arena) cudaFree(b->arena);
         if (b->d_jobs) cudaFree(b->d_jobs);
         if (b->d_meta) cudaFree(b->d_meta);
+        if (b->seen) cudaFreeHost(b->seen);
         if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
         delete b;
         return rc;
@@ -366,6 +372,9 @@ int vjb_batch_create(vjb_batch **out, int device, void *cuda_stream, int64_t tab
         cudaMalloc(&b->d_meta, sizeof(BatchMeta)) != cudaSuccess)
         return bail(fail(VJB_ENOMEM, "batch job table"));
     cudaMemset(b->d_meta, 0, sizeof(BatchMeta));
+    if (cudaHostAlloc(&b->seen, sizeof(BatchSeen), cudaHostAllocMapped) != cudaSuccess)
+        return bail(fail(VJB_ENOMEM, "batch round record"));
+    memset(b->seen, 0, sizeof(BatchSeen));
     const int rc = batch_encode_maps(b);
     if (rc) return bail(rc);
     b->free_list.emplace_back(0, b->arena_lines);
@@ -382,6 +391,7 @@ void vjb_batch_destroy(vjb_batch *b) {
     dfree(b->arena);
     dfree(b->d_jobs);
     dfree(b->d_meta);
+    if (b->seen) cudaFreeHost(b->seen);
     dfree(b->d_items);
     for (auto &t : b->ev_pending) b->ev_free.push_back(t);
     for (auto &t : b->ev_free)
@@ -797,12 +807,12 @@ ServerReq *req_of_slot(vjb_server *s, int32_t slot) {
 }
 
 // Jobs that reached their round count or stopped leave the batch.
-int server_retire(vjb_server *s, const std::vector<RoundState> &st) {
+int server_retire(vjb_server *s, const std::vector<JobSeen> &st) {
     vjb_batch *b = s->b;
     std::vector<BatchSlot> keep;
     for (size_t k = 0; k < b->slots.size(); ++k) {
         const BatchSlot &sl = b->slots[k];
-        const RoundState &rs = st[k];
+        const JobSeen &rs = st[k];
         const bool done = rs.flags || rs.status != VJB_OK || rs.rounds >= sl.round_target;
         if (!done) {
             keep.push_back(sl);
@@ -964,7 +974,7 @@ int vjb_server_step(vjb_server *s, int32_t max_rounds, int32_t *rounds_run) {
     int ran = 0;
     for (; ran < max_rounds; ++ran) {
         int want = 0;
-        std::vector<RoundState> st;
+        std::vector<JobSeen> st;
         int rc = batch_rounds_wanted(b, &want, &st);
         if (rc) return rc;
         rc = server_retire(s, st);
@@ -994,7 +1004,7 @@ int vjb_server_step(vjb_server *s, int32_t max_rounds, int32_t *rounds_run) {
     // retire what the last round finished
     {
         int want = 0;
-        std::vector<RoundState> st;
+        std::vector<JobSeen> st;
         int rc = batch_rounds_wanted(b, &want, &st);
         if (rc) return rc;
         rc = server_retire(s, st);

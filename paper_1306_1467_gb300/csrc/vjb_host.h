@@ -71,6 +71,15 @@ struct PendingRound {
 // Both library units work in the vjb names.
 using namespace vjb;
 
+namespace vjb {
+// What the host reads after a round: the round state and the last stump, one
+// device block and one copy.
+struct RoundRecord {
+    RoundState rs;
+    vjb_stump last;
+};
+}  // namespace vjb
+
 // One training context (the C ABI's vjb_ctx): its device buffers and state.
 struct vjb_ctx {
     int device = 0;
@@ -99,8 +108,11 @@ struct vjb_ctx {
     uint8_t *d_miss = nullptr;
     int32_t *d_scratch = nullptr;  // table preparation: check state and listed rows
     double *d_partials = nullptr;
-    RoundState *d_rs = nullptr;
+    RoundState *d_rs = nullptr;      // the round state in a RoundRecord, its last stump after it
     vjb_stump *d_stumps = nullptr, *d_last = nullptr;
+    // the record as of the last read, while nothing has changed it since
+    RoundRecord seen{};
+    bool seen_now = false;
     vjb_round_diag *d_diag = nullptr;
     int stump_cap = 0;
     int bmin_cap = 0;
@@ -146,7 +158,10 @@ struct vjb_ctx {
         rows_external = false;
         dfree(d_w); dfree(d_v); dfree(d_wtmp); dfree(d_ferr); dfree(d_bmin); dfree(d_cand);
         dfree(d_cand_ids); dfree(d_miss); dfree(d_partials); dfree(d_scratch);
-        dfree(d_rs); dfree(d_stumps); dfree(d_last); dfree(d_diag); dfree(d_cls);
+        dfree(d_rs); dfree(d_stumps); dfree(d_diag);
+        d_last = nullptr;
+        seen_now = false;
+        dfree(d_cls);
         cls_bytes = 0;
         stump_cap = bmin_cap = 0;
         feats.clear();

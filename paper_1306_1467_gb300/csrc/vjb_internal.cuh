@@ -203,12 +203,22 @@ struct BatchMeta {
     int64_t cta_start[kMaxScreenCtas + 1];
 };
 
+// What the host needs to know after a batched round, written by its last kernel
+// into mapped host memory (a copy per job and one of the counters took 60 to
+// 100 us a round of a server).
+constexpr int kMaxBatchJobs = 256;
+struct JobSeen {
+    int32_t status, rounds, flags, pad;
+};
+struct BatchSeen {
+    int32_t flags, pad[3];
+    JobSeen job[kMaxBatchJobs];
+};
+
 // A search work item: features [f0, f1) of one job.
 struct WorkItem {
     int32_t job, f0, f1, pad;
 };
-
-constexpr int kMaxBatchJobs = 256;
 
 struct SearchShape {
     int warps;        // consumer warps per CTA
@@ -272,6 +282,7 @@ cudaError_t launch_bshortlist(const JobDesc *jobs, BatchMeta *meta, int grid, cu
 cudaError_t launch_brescan(const JobDesc *jobs, BatchMeta *meta, int grid, cudaStream_t st);
 cudaError_t launch_bupdate_a(const JobDesc *jobs, BatchMeta *meta, int grid, cudaStream_t st);
 cudaError_t launch_bupdate_b(const JobDesc *jobs, BatchMeta *meta, int grid, cudaStream_t st);
+cudaError_t launch_bend(const JobDesc *jobs, const BatchMeta *meta, BatchSeen *seen, cudaStream_t st);
 size_t bscreen_smem_bytes(const SearchShape &s, int max_words);
 cudaError_t set_bscreen_smem_limit(int bytes);
 int update_grid(int n);

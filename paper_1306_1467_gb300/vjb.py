@@ -13,6 +13,8 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
+from operator import itemgetter
 
 import numpy as np
 
@@ -46,6 +48,30 @@ class Stump(C.Structure):
         return dict(feature=int(self.feature), threshold=int(self.threshold),
                     polarity=int(self.polarity), split=int(self.split), error=float(self.error),
                     beta=float(self.beta), alpha=float(self.alpha))
+
+
+_STUMP_KEYS = tuple(k for k, _ in Stump._fields_)
+_STUMP_ROW = struct.Struct("iiiiddd")  # a Stump's layout, for lists of them
+_stump_values = itemgetter(*_STUMP_KEYS)
+
+
+def _stump_dicts(arr, count: int) -> list:
+    """The first ``count`` Stumps of an array as dicts."""
+    rows = memoryview(arr).cast("B")[: count * _STUMP_ROW.size]
+    return [dict(zip(_STUMP_KEYS, v)) for v in _STUMP_ROW.iter_unpack(rows)]
+
+
+def _stump_array(stumps):
+    """Stump dicts as an array."""
+    try:
+        return (Stump * max(len(stumps), 1)).from_buffer_copy(
+            b"".join([_STUMP_ROW.pack(*v) for v in map(_stump_values, stumps)]) or bytes(_STUMP_ROW.size))
+    except struct.error:  # a value the packed form refuses: as ctypes takes it
+        arr = (Stump * len(stumps))()
+        for t, s in enumerate(stumps):
+            for k in _STUMP_KEYS:
+                setattr(arr[t], k, s[k])
+        return arr
 
 
 class Info(C.Structure):
@@ -303,7 +329,7 @@ class Trainer:
         arr = (Stump * max(int(T), 1))()
         done = C.c_int32(0)
         st = self._check(self._lib.vjb_train_strong(self._h, int(T), arr, C.byref(done)))
-        return st, [arr[t].as_dict() for t in range(done.value)]
+        return st, _stump_dicts(arr, done.value)
 
     def force_stump(self, feature: int, threshold: int, polarity: int):
         s = Stump()
@@ -362,10 +388,7 @@ class Trainer:
         (dicts as returned by train_round / train_strong)."""
         px = np.ascontiguousarray(pixels, np.uint8)
         n = px.shape[0]
-        arr = (Stump * max(len(stumps), 1))()
-        for t, s in enumerate(stumps):
-            for k, _ in Stump._fields_:
-                setattr(arr[t], k, s[k])
+        arr = _stump_array(stumps)
         lab = np.zeros(n, np.uint8)
         sc = np.zeros(n, np.float64)
         self._check(self._lib.vjb_classify(self._h, _ptr(px), n, arr, len(stumps), _ptr(lab), _ptr(sc)))
@@ -485,7 +508,7 @@ class Batch:
         done, _ = self.job_state(job_id)
         arr = (Stump * max(done, 1))()
         self._check(self._lib.vjb_batch_get_stumps(self._h, int(job_id), 0, done, arr))
-        return [arr[t].as_dict() for t in range(done)]
+        return _stump_dicts(arr, done)
 
     def get_weights(self, job_id: int) -> np.ndarray:
         out = np.zeros(self.jobs[int(job_id)], np.float32)
@@ -580,7 +603,7 @@ class Server:
         w = np.zeros(n, np.float32)
         st = self._check(self._lib.vjb_server_result(self._h, int(rid), arr, rounds, _ptr(w)))
         done = self.request(rid)["rounds_done"]
-        return st, [arr[t].as_dict() for t in range(done)], w
+        return st, _stump_dicts(arr, done), w
 
     def release(self, rid: int):
         self._check(self._lib.vjb_server_release(self._h, int(rid)))
