@@ -275,6 +275,16 @@ static size_t noalloc_smem_bytes(const SearchShape &s) {
     return b;
 }
 
+// Predicated running max/min: update only where `flag` is set (a valid split).
+__device__ __forceinline__ void minmax_if(uint32_t flag, float a, float &mx, float &mn) {
+    asm("{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %2, 0;\n\t"
+        "@p max.f32 %0, %0, %3;\n\t"
+        "@p min.f32 %1, %1, %3;\n\t}"
+        : "+f"(mx), "+f"(mn)
+        : "r"(flag), "f"(a));
+}
+
 // One stage of a row.  The lane's 32 entries are two pieces of 16 summed from
 // zero side by side; their largest and smallest prefixes at valid splits are
 // placed on the row by an FP32 scan of the 32 lanes' totals and the
@@ -288,7 +298,8 @@ static size_t noalloc_smem_bytes(const SearchShape &s) {
 // never waited.  A scan per 1,024 entries instead of per 512, no clamps at the
 // gathers, the weights staged behind the first copies and 16 warps instead of
 // 8: 452 -> 281 us a call there (3.46 TB/s).  Weights first in shared memory
-// (constant gather addresses) were slower, 299 us.
+// (constant gather addresses) were slower, 299 us, and so were entries taken two
+// at a time as in k_screen (scan_two), 305 us.
 __device__ __forceinline__ void screen_stage_plain(uint32_t sbase, int lane, const float *__restrict__ sv, float &chi,
                                                    float &clo, float &MX, float &MN) {
     // chunk c of line l is stored at chunk c ^ (l mod 8) (128-byte swizzle):

@@ -26,14 +26,35 @@ __device__ __forceinline__ void stage_weights(float *sv, const float *v, int wor
     for (int i = threadIdx.x; i < n4; i += blockDim.x) sv4[i] = __ldg(v4 + i);
 }
 
-// Predicated running max/min: update only where `flag` is set (a valid split).
-__device__ __forceinline__ void minmax_if(uint32_t flag, float a, float &mx, float &mn) {
+// The prefix a = before + g where `flag` is set (a valid split), else `kept`
+// as it was.
+__device__ __forceinline__ void keep_if(uint32_t flag, float before, float g, float &kept) {
     asm("{\n\t.reg .pred p;\n\t"
-        "setp.ne.u32 p, %2, 0;\n\t"
-        "@p max.f32 %0, %0, %3;\n\t"
-        "@p min.f32 %1, %1, %3;\n\t}"
-        : "+f"(mx), "+f"(mn)
-        : "r"(flag), "f"(a));
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "@p add.rn.f32 %0, %2, %3;\n\t}"
+        : "+f"(kept)
+        : "r"(flag), "f"(before), "f"(g));
+}
+
+// Two neighbouring entries of a piece: their weights join the running sum a,
+// and the prefix after each, where its flag marks a valid split, the running
+// extremes.  `even` and `odd` hold the last valid prefix at an even and at an
+// odd position (an invalid split leaves one that has counted already; NaN
+// while there is none, which a max or min passes over), so that one
+// three-input max and one min take both: half the instructions of a
+// predicated max and min an entry, on the pipe (ALU) that is the busiest after
+// shared memory.  k_screen at 24x24 / 15,000 samples 0.745 -> 0.729 ms, 8,000
+// 0.421 -> 0.411, 4,096 0.223 -> 0.219, 10,963 0.559 -> 0.556, 2,003 0.125 ->
+// 0.1235; 32x32 / 5,003 0.855 -> 0.859.  The kept prefix is added a second
+// time rather than copied: a copy waits for the sum (0.748).
+__device__ __forceinline__ void scan_two(uint32_t flag_even, uint32_t flag_odd, float g_even, float g_odd, float &a,
+                                         float &even, float &odd, float &mx, float &mn) {
+    keep_if(flag_even, a, g_even, even);
+    a += g_even;
+    keep_if(flag_odd, a, g_odd, odd);
+    a += g_odd;
+    mx = fmaxf(mx, fmaxf(even, odd));
+    mn = fminf(mn, fminf(even, odd));
 }
 
 // U pieces of CR chunk rows of a stage (8 entries per lane per chunk row),
@@ -66,21 +87,20 @@ __device__ __forceinline__ void scan_pieces(uint32_t sbase, int t0, int lane, co
             g[u][2 * j] = sv[wd[u][j] & kIndexMask];  // even position: word | flag << 15
             g[u][2 * j + 1] = sv[wd[u][j] >> 17];      // odd position: (word << 1 | flag) << 16
         }
-    float a[U], mx[U], mn[U];
+    float a[U], mx[U], mn[U], even[U], odd[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         a[u] = 0.f;
         mx[u] = -INFINITY;
         mn[u] = INFINITY;
+        even[u] = odd[u] = __int_as_float(0x7fc00000);  // NaN
     }
 #pragma unroll
-    for (int j = 0; j < E; ++j)
+    for (int j = 0; j < E / 2; ++j)
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            a[u] += g[u][j];
-            const uint32_t fl = (j & 1) ? (wd[u][j >> 1] & 0x10000u) : (wd[u][j >> 1] & 0x8000u);
-            minmax_if(fl, a[u], mx[u], mn[u]);
-        }
+        for (int u = 0; u < U; ++u)
+            scan_two(wd[u][j] & 0x8000u, wd[u][j] & 0x10000u, g[u][2 * j], g[u][2 * j + 1], a[u], even[u], odd[u],
+                     mx[u], mn[u]);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         bmx = fmaxf(bmx, ahi + (alo + mx[u]));
