@@ -485,10 +485,12 @@ static cudaError_t launch_sort_ipt(const int32_t *ii_t, int ii_stride, int w, co
 // ALU 53%, 132 instructions an item).  Ranking with one ballot per digit bit,
 // the form before, was ALU bound at 223 instructions an item.  Tables in all,
 // then -> with atomics -> with gaps between the finished runs (kRunGap) and the
-// samples of one copy placed first:
-//   24x24 / 2,003   6.04 ->  2.90 ->  2.54 ms    32x32 / 5,003   31.9 -> 20.0 -> 17.1
-//   24x24 / 10,963  16.4 -> 12.9  -> 12.3         24x24 / 15,000  20.9 -> 16.1 -> 15.7
-//   24x24 / 18,300  34.4 -> 26.0  -> 21.8
+// samples of one copy placed first -> values eight windows a load, counts in batches:
+//   24x24 / 2,003   6.04 ->  2.90 ->  2.54 ->  2.54 ms
+//   32x32 / 5,003   31.9 ->  20.0 ->  17.1 ->  16.8
+//   24x24 / 10,963  16.4 ->  12.9 ->  12.3 ->  11.6
+//   24x24 / 15,000  20.9 ->  16.1 ->  15.8 ->  15.0
+//   24x24 / 18,300  34.4 ->  26.0 ->  21.9 ->  21.0
 //
 // Threads per CTA grow with the row (128 up to 4,096 samples, 256 up to 8,192,
 // 512 up to 16,384), 1,024 threads an SM in all: small CTAs leave other rows
@@ -546,40 +548,47 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
     const DevFeature d = feat[f0 + blockIdx.x];
 
     // the feature on every window (K2's arithmetic), four windows per thread
-    // and corner load.  Boxes of at most kNarrowArea pixels come from the
-    // integral images modulo 2^16, two windows to a 32-bit word (half the
-    // bytes, and the corners are added two windows at a time); they are kept
-    // as 16-bit offsets from the type's smallest possible value.
+    // and point.  Boxes of at most kNarrowArea pixels come from the
+    // integral images modulo 2^16, eight windows a load and two to a 32-bit
+    // word (half the bytes, and the points are added two windows at a time);
+    // they are kept as 16-bit offsets from the type's smallest possible value.
     const bool narrow = ii16 && d.w * d.h <= kNarrowArea;
     uint16_t *val16 = reinterpret_cast<uint16_t *>(skey);
     int32_t lo = INT_MAX, hi = INT_MIN;
     if (narrow) {
         uint32_t lo2 = 0xffffffffu, hi2 = 0u;
-        for (int q = threadIdx.x; 4 * q < n; q += TH) {
-            const int p = 4 * q;
-            uint2 x = haar_offsets4(ii16, ii_stride, w, d.type, d.x, d.y, d.w, d.h, p);
-            if (p + 4 > n) {  // past the last sample: repeat the last one's
-                if (p + 1 >= n) x.x = (x.x & 0xffffu) * 0x10001u;
-                if (p + 2 >= n) x.y = (x.x >> 16) * 0x10001u;
-                else x.y = (x.y & 0xffffu) * 0x10001u;
+        haar_rows_narrow<TH>(ii16, ii_stride, w, d.type, d.x, d.y, d.w, d.h, n, [&](int q, uint4 x) {
+            const int left = n - 8 * q;  // at least 1
+            if (left < 8) {  // past the last sample: repeat the window before, word by word
+                auto half = [](uint32_t a) { return (a & 0xffffu) * 0x10001u; };
+                if (left == 1) x.x = half(x.x);
+                if (left <= 2) x.y = (x.x >> 16) * 0x10001u;
+                if (left == 3) x.y = half(x.y);
+                if (left <= 4) x.z = (x.y >> 16) * 0x10001u;
+                if (left == 5) x.z = half(x.z);
+                if (left <= 6) x.w = (x.z >> 16) * 0x10001u;
+                if (left == 7) x.w = half(x.w);
             }
-            reinterpret_cast<uint2 *>(skey)[q] = x;
-            lo2 = __vminu2(lo2, __vminu2(x.x, x.y));
-            hi2 = __vmaxu2(hi2, __vmaxu2(x.x, x.y));
-        }
+            reinterpret_cast<uint4 *>(skey)[q] = x;
+            lo2 = __vminu2(__vminu2(lo2, __vminu2(x.x, x.y)), __vminu2(x.z, x.w));
+            hi2 = __vmaxu2(__vmaxu2(hi2, __vmaxu2(x.x, x.y)), __vmaxu2(x.z, x.w));
+        });
         lo = (int32_t)min(lo2 & 0xffffu, lo2 >> 16);
         hi = (int32_t)max(hi2 & 0xffffu, hi2 >> 16);
     } else {
-        for (int q = threadIdx.x; 4 * q < n; q += TH) {
-            const int p = 4 * q;
-            const int4 x = haar_value4(ii_t, ii_stride, w, d.type, d.x, d.y, d.w, d.h, p);
-            reinterpret_cast<uint4 *>(skey)[q] = make_uint4((uint32_t)x.x, (uint32_t)x.y, (uint32_t)x.z, (uint32_t)x.w);
-            lo = min(lo, x.x);
-            hi = max(hi, x.x);
-            if (p + 1 < n) { lo = min(lo, x.y); hi = max(hi, x.y); }
-            if (p + 2 < n) { lo = min(lo, x.z); hi = max(hi, x.z); }
-            if (p + 3 < n) { lo = min(lo, x.w); hi = max(hi, x.w); }
-        }
+        haar_rows<TH, int4>(
+            ii_t, ii_stride, w, d.type, d.x, d.y, d.w, d.h, n,
+            [](int4 a, int4 b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); },
+            [&](int q, int4 pos, int4 neg) {
+                const int p = 4 * q;
+                const int4 x = make_int4(pos.x - neg.x, pos.y - neg.y, pos.z - neg.z, pos.w - neg.w);
+                reinterpret_cast<int4 *>(skey)[q] = x;
+                lo = min(lo, x.x);
+                hi = max(hi, x.x);
+                if (p + 1 < n) { lo = min(lo, x.y); hi = max(hi, x.y); }
+                if (p + 2 < n) { lo = min(lo, x.z); hi = max(hi, x.z); }
+                if (p + 3 < n) { lo = min(lo, x.w); hi = max(hi, x.w); }
+            });
     }
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
@@ -618,11 +627,18 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
         const uint32_t per_run = shift + D >= bits ? 0xffffffffu / (uint32_t)run + 1u : 0u;
         for (int k = lane; k < (1 << D); k += 32) own[k] = 0u;
         __syncwarp();
+        // (eight items are read, then counted: an item's read would wait for the
+        // add before it; tables at 24x24 / 10,963 11.9 -> 11.6 ms)
         auto count = [&](auto whole) {
+            constexpr int BATCH = 8;
 #pragma unroll
-            for (int j = 0; j < IPT; ++j) {
-                const uint32_t at = (digit(pos0 + 32 * j, sh) & dmask) | own32;
-                shared_add(decltype(whole)::value || j < mine ? at : spare32, 1u);
+            for (int j0 = 0; j0 < IPT; j0 += BATCH) {
+                uint32_t at[BATCH];
+#pragma unroll
+                for (int u = 0; u < BATCH && j0 + u < IPT; ++u) at[u] = (digit(pos0 + 32 * (j0 + u), sh) & dmask) | own32;
+#pragma unroll
+                for (int u = 0; u < BATCH && j0 + u < IPT; ++u)
+                    shared_add(decltype(whole)::value || j0 + u < mine ? at[u] : spare32, 1u);
             }
         };
         if (all_mine) count(std::true_type{});
