@@ -481,28 +481,39 @@ static cudaError_t launch_sort_ipt(const int32_t *ii_t, int ii_stride, int w, co
 // one 16-byte chunk per thread.
 //
 // What bounds it: shared memory (16x16 / 15,000 under ncu: its pipe 66% busy, 37
-// wavefronts per 32 items, half of them the atomics' bank conflicts; issue 49%,
-// ALU 53%, 132 instructions an item).  Ranking with one ballot per digit bit,
-// the form before, was ALU bound at 223 instructions an item.  Tables in all,
-// then -> with atomics -> with gaps between the finished runs (kRunGap) and the
-// samples of one copy placed first -> values eight windows a load, counts in batches:
-//   24x24 / 2,003   6.04 ->  2.90 ->  2.54 ->  2.54 ms
-//   32x32 / 5,003   31.9 ->  20.0 ->  17.1 ->  16.8
-//   24x24 / 10,963  16.4 ->  12.9 ->  12.3 ->  11.6
-//   24x24 / 15,000  20.9 ->  16.1 ->  15.8 ->  15.0
-//   24x24 / 18,300  34.4 ->  26.0 ->  21.9 ->  21.0
+// wavefronts per 32 items, half of them the atomics' bank conflicts) and the
+// barriers between phases that use it unevenly.  Ranking with one ballot per
+// digit bit, the form before, was ALU bound at 223 instructions an item.
+// Tables in all, then -> with atomics -> with gaps between the finished runs
+// (kRunGap) and the samples of one copy placed first -> values eight windows a
+// load, counts in batches -> smaller CTAs, and rows whose last runs are short
+// chosen and written like whole ones:
+//   24x24 / 2,003   6.04 ->  2.90 ->  2.54 ->  2.54 ->  2.27 ms
+//   32x32 / 5,003   31.9 ->  20.0 ->  17.1 ->  16.8 ->  15.6
+//   24x24 / 10,963  16.4 ->  12.9 ->  12.3 ->  11.6 ->  10.3
+//   24x24 / 15,000  20.9 ->  16.1 ->  15.8 ->  15.0 ->  13.8
+//   24x24 / 18,300  34.4 ->  26.0 ->  21.9 ->  21.0 ->  19.1
 //
-// Threads per CTA grow with the row (128 up to 4,096 samples, 256 up to 8,192,
-// 512 up to 16,384), 1,024 threads an SM in all: small CTAs leave other rows
-// to run while one waits at a barrier.  From 16,385 to 20,480 samples two CTAs
-// of 640 threads still fit an SM (18,300: 26.0 ms, 29.9 with one CTA of 1,024);
-// above, one of 1,024.
+// Threads per CTA: few, with as many items each as the registers hold (128
+// threads up to 4,096 samples, 256 up to 15,360, 384 with two CTAs an SM up to
+// 20,736, then 512).  Every warp has counters of its own to clear and scan, and
+// more and smaller CTAs leave other rows to run while one waits at a barrier:
+// 256 threads of 40 to 60 items, three CTAs an SM, against 512 of 20 to 30, two:
+// 10,000 samples 11.24 -> 9.74 ms, 13,000 13.36 -> 11.9, 15,000 15.0 -> 14.1; 384
+// of 48 against 640 of 30: 18,300 21.0 -> 19.0; 512 of 48 and 64 against 1,024 of
+// 24 and 32: 24,000 13.3 -> 12.4, 32,766 12.9 -> 12.3.  The other way round costs:
+// 512 threads of 16 at 8,000 8.6 against 7.6 ms, 640 of 24 at 15,000 15.6 against
+// 15.0; so do too few warps: 128 of 40 at 5,003 17.3 against 16.7 ms, 192 of 40 at
+// 7,148 7.14 against 6.91.
 //
 // Measured and dropped: one pass with a counter per value for spans up to 14
 // bits (one warp ranking a row in order waits its turn behind the other CTA's
 // warps: 16.9 ms at 15,000); buckets filled in any order and put right by
 // counting or by insertion (28.7 ms); predicated atomics for the last warp's
-// missing items (the compiler wraps each in a branch: 158 instructions).
+// missing items (the compiler wraps each in a branch: 158 instructions); the
+// row filled up to whole groups of 32 items and whole groups skipped (the
+// batches' branches cost more registers: 15,000 13.8 -> 14.1, 3,300 3.5 -> 3.75,
+// though 4,090 3.83 -> 3.59).
 constexpr int kPkDigitBits = 8;
 // Words between the 32 lane runs of a finished row in shared memory: runs are a
 // multiple of 8 words long, and without a gap the reads of one place in every
@@ -523,8 +534,16 @@ __device__ __forceinline__ uint32_t shared_take(uint32_t addr) {
     return old;
 }
 
+// CTAs an SM by registers: a thread holds its IPT items and about 20 values
+// more.  (40 registers for 16 items and 48 for 20 spill a little, outside the
+// passes, and are still better than fewer CTAs: 2,003 2.53 -> 2.49 ms, 32x32 /
+// 5,003 16.84 -> 16.73.)
+constexpr int packed_ctas(int ipt, int th) {
+    return 65536 / (th * (ipt <= 16 ? 40 : ipt <= 20 ? 48 : ipt <= 32 ? 64 : ipt <= 48 ? 72 : 80));
+}
+
 template <int IPT, int TH>
-__global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
+__global__ void __launch_bounds__(TH, packed_ctas(IPT, TH))
     k_sort_rows_packed(const int32_t *__restrict__ ii_t, const uint16_t *__restrict__ ii16, int ii_stride, int w,
                        const DevFeature *__restrict__ feat, int64_t f0, WeightLayout L,
                        uint16_t *__restrict__ rows, int npad, int32_t *ovf, int32_t *stat) {
@@ -646,7 +665,7 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
         __syncthreads();
         // first positions, by digit, then warp: a thread takes digit q * TH +
         // tid of every warp's counters
-        constexpr int ROUNDS = kPkRadix / TH > 0 ? kPkRadix / TH : 1;
+        constexpr int ROUNDS = (kPkRadix + TH - 1) / TH;
         uint32_t pre[ROUNDS];
 #pragma unroll
         for (int q = 0; q < ROUNDS; ++q) {
@@ -740,20 +759,26 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
         };
         if (threadIdx.x == 0) mm[0] = 0;
         __syncthreads();
+        // Of a group's 32 entries every group has `whole`, and those below row
+        // position n one more: a loop of that length diverges, and rolled it
+        // took as long again as the rest (2,003 samples: tables 2.49 -> 2.33 ms,
+        // 32x32 / 5,003 16.7 -> 15.8).
+        const int whole = n / run;
         auto choose = [&](auto partial) {
             for (int g = threadIdx.x; g < run; g += TH) {
                 uint32_t m1 = 0u, m2 = 0u, m3 = 0u, mask = 0u;
-                const int kend = min(32, (n - g + run - 1) / run);  // entries k * run + g < n
                 const uint32_t *first = skey + g;
+                const int kend = whole + (whole * run + g < n ? 1 : 0);  // entries k * run + g < n
                 auto put = [&](uint32_t to) {
                     m3 |= m2 & to;
                     m2 |= m1 & to;
                     m1 |= to;
                 };
-                auto entry = [&](int k) {
+                auto entry = [&](int k, bool there) {
                     const uint32_t x = first[k * pitch];
                     uint32_t a, b;
                     bank_bits(x, a, b);
+                    if (!there) a = b = 0u;
                     if (decltype(partial)::value && (int)(x & imask) >= L.nb) a = b = 0u;  // placed before
                     // bank b is less loaded if it has no entry and a has one,
                     // or has one and a has two; without branches
@@ -770,25 +795,31 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
                         : "r"(m1), "r"(m2), "r"(a), "r"(b), "r"(1u << k));
                     put(to);
                 };
-                if (decltype(partial)::value) {
-                    // the samples with one copy first: those with two fill the gaps
-#pragma unroll 8
-                    for (int k = 0; k < kend; ++k) {
-                        const uint32_t x = first[k * pitch];
-                        put((int)(x & imask) >= L.nb ? __funnelshift_l(0u, 1u, x) : 0u);
+                // eight entries at a time; past the row's end (position k * run +
+                // g, in the last runs only) an entry counts nothing
+                auto entries = [&](auto each) {
+                    for (int k0 = 0; k0 < 32; k0 += 8) {
+                        if (k0 + 8 <= whole) {
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) each(k0 + u, true);
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) each(k0 + u, k0 + u < kend);
+                        }
                     }
-                }
-                if (kend == 32) {
-#pragma unroll 8
-                    for (int k = 0; k < 32; ++k) entry(k);
-                } else {
-                    for (int k = 0; k < kend; ++k) entry(k);
-                    put(1u << (n & 31));  // the padding word, read as a broadcast
-                }
+                };
+                if (decltype(partial)::value)
+                    // the samples with one copy first: those with two fill the gaps
+                    entries([&](int k, bool there) {
+                        const uint32_t x = first[k * pitch];
+                        put(there && (int)(x & imask) >= L.nb ? __funnelshift_l(0u, 1u, x) : 0u);
+                    });
+                entries(entry);
+                if (kend < 32) put(1u << (n & 31));  // the padding word, read as a broadcast
                 gchoice[g] = mask;
-                // (rows above 20,480 samples: so few entries have two copies that
+                // (rows above 20,736 samples: so few entries have two copies that
                 // refining buys no search time; 24,000: 5 us for 2.9 ms)
-                if (m3 && (TH < 1024 || !decltype(partial)::value)) {
+                if (m3 && (NP <= 54 * 384 || !decltype(partial)::value)) {
                     const int q = atomicAdd(&mm[0], 1);
                     reinterpret_cast<uint4 *>(rlist)[q] = make_uint4((uint32_t)g, m1, m2, m3);
                 }
@@ -861,7 +892,10 @@ __global__ void __launch_bounds__(TH, TH == 640 ? 2 : 1024 / TH)
         }
         uint32_t wv[kChunkElems / 2];
         const uint32_t lanebit = 1u << k;
-        if (p0 + kChunkElems < n) {  // the row goes on after the chunk
+        if (p0 >= n) {  // padding, at the end of the last lane run: one lane of a warp (2,003: 2.33 -> 2.27 ms)
+            const uint32_t two = make_entry(n, false, 0) | make_entry(n, false, 1) << 16;
+            wv[0] = wv[1] = wv[2] = wv[3] = two;
+        } else if (p0 + kChunkElems < n) {  // the row goes on after the chunk
 #pragma unroll
             for (int j = 0; j < kChunkElems; ++j) {
                 const uint32_t i = cp[j] & imask;
@@ -966,19 +1000,18 @@ cudaError_t launch_sort_rows(const int32_t *ii_t, const uint16_t *ii16, int ii_s
     VJB_PK_CASE(24, 256)
     VJB_PK_CASE(28, 256)
     VJB_PK_CASE(32, 256)
-    VJB_PK_CASE(20, 512)
-    VJB_PK_CASE(22, 512)
-    VJB_PK_CASE(24, 512)
-    VJB_PK_CASE(26, 512)
-    VJB_PK_CASE(28, 512)
-    VJB_PK_CASE(30, 512)
-    VJB_PK_CASE(32, 512)
-    VJB_PK_CASE(28, 640)
-    VJB_PK_CASE(30, 640)
-    VJB_PK_CASE(32, 640)
-    VJB_PK_CASE(24, 1024)
-    VJB_PK_CASE(28, 1024)
-    VJB_PK_CASE(32, 1024)
+    VJB_PK_CASE(36, 256)
+    VJB_PK_CASE(40, 256)
+    VJB_PK_CASE(44, 256)
+    VJB_PK_CASE(48, 256)
+    VJB_PK_CASE(52, 256)
+    VJB_PK_CASE(56, 256)
+    VJB_PK_CASE(60, 256)
+    VJB_PK_CASE(44, 384)
+    VJB_PK_CASE(48, 384)
+    VJB_PK_CASE(54, 384)
+    VJB_PK_CASE(48, 512)
+    VJB_PK_CASE(64, 512)
     e = cudaErrorInvalidValue;
 #undef VJB_PK_CASE
     if (e != cudaSuccess) return e;

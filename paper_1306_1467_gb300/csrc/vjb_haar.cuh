@@ -1,5 +1,5 @@
 // Haar feature values (Sec. 2.1-2.2) from the point-major integral images:
-// one window, all windows of a row at four a load, and the narrow-box form
+// one window, all windows of a row, several a load, and the narrow-box form
 // from the integral images modulo 2^16.
 #pragma once
 
