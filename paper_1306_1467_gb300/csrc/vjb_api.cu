@@ -352,7 +352,9 @@ int load_common(vjb_ctx *c, const uint8_t *pixels, const uint8_t *labels, int32_
         CK(cudaMalloc(&c->d_wtmp, sizeof(float) * n));
         c->lay = make_layout(n, true);
         CK(cudaMalloc(&c->d_v, sizeof(float) * c->lay.words));
-        CK(cudaMemset(c->d_v, 0, sizeof(float) * c->lay.words));
+        // on the context's stream: on the default stream, which a non-blocking one
+        // does not wait for, the zeros could come after the weights
+        CK(cudaMemsetAsync(c->d_v, 0, sizeof(float) * c->lay.words, c->stream));
         CK(cudaMalloc(&c->d_miss, (size_t)n));
         CK(cudaMalloc(&c->d_partials, sizeof(double) * 3 * kUpdateMaxCtas));
         CK(cudaMalloc(&c->d_rs, sizeof(RoundRecord)));

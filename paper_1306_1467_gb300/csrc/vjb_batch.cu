@@ -371,7 +371,8 @@ int vjb_batch_create(vjb_batch **out, int device, void *cuda_stream, int64_t tab
     if (cudaMalloc(&b->d_jobs, sizeof(JobDesc) * kMaxBatchJobs) != cudaSuccess ||
         cudaMalloc(&b->d_meta, sizeof(BatchMeta)) != cudaSuccess)
         return bail(fail(VJB_ENOMEM, "batch job table"));
-    cudaMemset(b->d_meta, 0, sizeof(BatchMeta));
+    if (cudaMemsetAsync(b->d_meta, 0, sizeof(BatchMeta), b->stream) != cudaSuccess)
+        return bail(fail(VJB_ECUDA, "batch job table"));
     if (cudaHostAlloc(&b->seen, sizeof(BatchSeen), cudaHostAllocMapped) != cudaSuccess)
         return bail(fail(VJB_ENOMEM, "batch round record"));
     memset(b->seen, 0, sizeof(BatchSeen));
