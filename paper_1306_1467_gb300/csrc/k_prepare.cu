@@ -480,7 +480,7 @@ static cudaError_t launch_sort_ipt(const int32_t *ii_t, int ii_stride, int w, co
 // Then the bank choice of the two weight copies and the run-interleaved write,
 // one 16-byte chunk per thread.
 //
-// What bounds it: shared memory (16x16 / 15,000 under ncu: its pipe 66% busy, 37
+// What bounds it: shared memory (16x16 / 15,000 under ncu: its pipe 74% busy, 37
 // wavefronts per 32 items, half of them the atomics' bank conflicts) and the
 // barriers between phases that use it unevenly.  Ranking with one ballot per
 // digit bit, the form before, was ALU bound at 223 instructions an item.
