@@ -782,6 +782,12 @@ int vjb_classify(vjb_ctx *c, const uint8_t *pixels, int32_t n, const vjb_stump *
         for (auto &ev : c->cls_ev)
             if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     }
+    if (e == cudaSuccess && parts > 1) {
+        // the copies come after what the caller has queued on the context's
+        // stream (its windows may still be on their way into pinned memory)
+        e = cudaEventRecord(c->cls_ev[0], c->stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(c->copy_stream, c->cls_ev[0], 0);
+    }
     if (e == cudaSuccess && T > 0) e = cudaMemcpyAsync(d_st, cs.data(), sizeof(ClassStump) * T, cudaMemcpyHostToDevice, c->stream);
     for (int k = 0; k < parts && e == cudaSuccess; ++k) {
         const int i0 = k * part, m = std::min(part, n - i0), buf = k & 1;
