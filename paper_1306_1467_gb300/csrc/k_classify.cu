@@ -96,17 +96,25 @@ __global__ void __launch_bounds__(kFusedThreads)
     }
 }
 
-bool classify_fits(int h, int w, int max_smem) {
+// Once per device, before the first launch (as set_integral_limits): what a CTA
+// may have in all, `max_smem`, less what the kernel holds anyway.
+cudaError_t set_classify_limits(int max_smem) {
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, k_classify_windows);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_classify_windows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                max_smem - (int)fa.sharedSizeBytes);
+}
+
+bool classify_fits(int h, int w) {
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, k_classify_windows) != cudaSuccess) return false;
-    return classify_words(h, w) * 4 + fa.sharedSizeBytes <= (size_t)max_smem;
+    return classify_words(h, w) * 4 <= (size_t)fa.maxDynamicSharedSizeBytes;
 }
 
 cudaError_t launch_classify_windows(const uint8_t *px, int n, int h, int w, const ClassStump *stumps, int T,
                                     double half_alpha, uint8_t *labels, double *scores, cudaStream_t st) {
     const size_t sm = classify_words(h, w) * 4;
-    cudaError_t e = cudaFuncSetAttribute(k_classify_windows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
     k_classify_windows<<<(n + kTileWindows - 1) / kTileWindows, kFusedThreads, sm, st>>>(px, n, h, w, stumps, T,
                                                                                         half_alpha, labels, scores);
     return cudaGetLastError();

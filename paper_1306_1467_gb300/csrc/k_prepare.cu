@@ -67,13 +67,19 @@ __global__ void __launch_bounds__(kIntegralThreads)
     }
 }
 
+constexpr size_t kIntegralSmem = 100 * 1024;  // at most: two CTAs an SM
+
+// Once per device, before the first launch: a kernel's limit on shared memory is
+// the same for every context and thread, so a launch must not set its own.
+cudaError_t set_integral_limits() {
+    return cudaFuncSetAttribute(k_integral, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIntegralSmem);
+}
+
 cudaError_t launch_integral(const uint8_t *px, int n, int h, int w, int32_t *ii_t, uint16_t *ii16,
                             int ii_stride, cudaStream_t st) {
     auto bytes = [&](int band) { return ((size_t)band * w * 32 + w * 32 + 32 * tile_stride(band * w)) * 4; };
-    int band = h;  // two CTAs an SM, or a row at a time (up to 255 pixels: 73 KB)
-    while (band > 1 && bytes(band) > 100 * 1024) --band;
-    cudaError_t e = cudaFuncSetAttribute(k_integral, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(band));
-    if (e != cudaSuccess) return e;
+    int band = h;  // or fewer rows, down to one at a time (up to 255 pixels: 73 KB)
+    while (band > 1 && bytes(band) > kIntegralSmem) --band;
     k_integral<<<(n + kTileWindows - 1) / kTileWindows, kIntegralThreads, bytes(band), st>>>(px, n, h, w, band, ii_t,
                                                                                             ii16, ii_stride);
     return cudaGetLastError();

@@ -476,6 +476,8 @@ int vjb_create(vjb_ctx **out, int device, void *cuda_stream) {
     }
     if (e == cudaSuccess) e = set_screen_smem_limit(c->max_smem);
     if (e == cudaSuccess) e = set_tail_limits();
+    if (e == cudaSuccess) e = set_integral_limits();
+    if (e == cudaSuccess) e = set_classify_limits(c->max_smem);
     if (e == cudaSuccess && cuda_stream) {
         c->stream = static_cast<cudaStream_t>(cuda_stream);
     } else if (e == cudaSuccess) {
@@ -755,7 +757,7 @@ int vjb_classify(vjb_ctx *c, const uint8_t *pixels, int32_t n, const vjb_stump *
     // memory and buffers allocated and freed).  Windows too large for shared
     // memory go through integral images in memory, whole.
     const size_t hw = (size_t)c->h * c->w;
-    const bool fused = classify_fits(c->h, c->w, c->max_smem);
+    const bool fused = classify_fits(c->h, c->w);
     const int part = fused ? (int)std::min<size_t>((size_t)(n + 31) / 32 * 32, std::max<size_t>(32, (kClassifyPartBytes / hw) / 32 * 32)) : n;
     const int parts = (n + part - 1) / part;
     const int stride = (n + 31) / 32 * 32;

@@ -234,6 +234,7 @@ WeightLayout make_layout(int n, bool allow_dual);
 // Launchers (each returns the launch error).
 cudaError_t launch_integral(const uint8_t *px, int n, int h, int w, int32_t *ii_t, uint16_t *ii16,
                             int ii_stride, cudaStream_t st);
+cudaError_t set_integral_limits();
 // One stump of a strong classifier as the kernels read it.
 struct ClassStump {
     DevFeature f;
@@ -243,7 +244,8 @@ struct ClassStump {
 cudaError_t launch_strong_classify(const int32_t *ii_t, int ii_stride, int n, int win_w, const ClassStump *stumps, int T,
                                    double half_alpha, uint8_t *labels, double *scores, cudaStream_t st);
 // The same from the pixels, for windows whose integral images fit shared memory.
-bool classify_fits(int h, int w, int max_smem);
+bool classify_fits(int h, int w);
+cudaError_t set_classify_limits(int max_smem);
 cudaError_t launch_classify_windows(const uint8_t *px, int n, int h, int w, const ClassStump *stumps, int T,
                                     double half_alpha, uint8_t *labels, double *scores, cudaStream_t st);
 // The feature list of a w x h window.
