@@ -981,9 +981,8 @@ int vjb_server_step(vjb_server *s, int32_t max_rounds, int32_t *rounds_run) {
         rc = server_retire(s, st);
         if (rc) return rc;
         if (want == 0) break;
-        int in_round = 0;
-        for (size_t k = 0; k < st.size(); ++k)
-            if (st[k].status == VJB_OK && !st[k].flags && st[k].rounds < b->slots[k].round_target) ++in_round;
+        // (`st` has the retired jobs' states too; those left all take part)
+        const int in_round = (int)b->slots.size();
         std::vector<ServerReq *> members;
         for (auto &sl : b->slots) {
             ServerReq *r = req_of_slot(s, sl.id);
