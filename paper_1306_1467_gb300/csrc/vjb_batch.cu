@@ -168,6 +168,7 @@ int batch_sync(vjb_batch *b) {
     m.total_ublocks = ubase;
     CK(cudaMemcpyAsync(b->d_meta, &m, sizeof m, cudaMemcpyHostToDevice, b->stream));
     CK(cudaStreamSynchronize(b->stream));
+    b->flags = 0;  // the counters are new: an error is reported until the jobs change
     b->dirty = false;
     return VJB_OK;
 }

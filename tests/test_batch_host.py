@@ -27,7 +27,7 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("case", ["step_counts"])
+@pytest.mark.parametrize("case", ["flags", "step_counts"])
 def test_batch_host(program, case):
     r = subprocess.run([program, case], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
