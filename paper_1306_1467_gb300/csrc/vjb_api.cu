@@ -234,7 +234,7 @@ int enqueue_search(vjb_ctx *c) {
 }
 
 int enqueue_tail(vjb_ctx *c) {
-    CK(launch_tail(job_desc(c), c->d_bmin, c->screen_grid, c->num_sms, c->stream));
+    CK(launch_tail(job_desc(c), c->d_bmin, c->screen_grid, c->plateau_clusters, c->stream));
     return VJB_OK;
 }
 
@@ -476,6 +476,7 @@ int vjb_create(vjb_ctx **out, int device, void *cuda_stream) {
     }
     if (e == cudaSuccess) e = set_screen_smem_limit(c->max_smem);
     if (e == cudaSuccess) e = set_tail_limits();
+    if (e == cudaSuccess) c->plateau_clusters = plateau_clusters();
     if (e == cudaSuccess) e = set_integral_limits();
     if (e == cudaSuccess) e = set_classify_limits(c->max_smem);
     if (e == cudaSuccess && cuda_stream) {

@@ -129,7 +129,7 @@ struct vjb_ctx {
     bool tmap_ok = false;
     SearchShape shape{12, 2, 1, 4, 32};
     bool shape_set = false;
-    int screen_grid = 0;
+    int screen_grid = 0, plateau_clusters = 1;
 
     // graph of one round; with timing on, of its search (graph) and of the
     // rest (graph2), launched with the timing events between them

@@ -262,9 +262,11 @@ cudaError_t launch_init_weights(const uint8_t *y, int faces, const WeightLayout 
 cudaError_t launch_screen(const CUtensorMap *tmap, const float *v, const WeightLayout &L,
                           int lines_per_row, int box_lines, int64_t nfeat, const SearchShape &shape,
                           int grid, RoundState *rs, float *ferr, float *bmin, cudaStream_t st);
-// What follows a plain round's search (two kernels), on a GPU of `sms` SMs.
-cudaError_t launch_tail(const JobDesc &J, const float *bmin, int nbmin, int sms, cudaStream_t st);
+// What follows a plain round's search (two kernels).  `clusters`: how many of the
+// long-list kernel's clusters the device runs at once (plateau_clusters).
+cudaError_t launch_tail(const JobDesc &J, const float *bmin, int nbmin, int clusters, cudaStream_t st);
 cudaError_t set_tail_limits();
+int plateau_clusters();
 // The update alone, with a host-given stump.
 cudaError_t launch_update_a(const JobDesc &J, cudaStream_t st);
 cudaError_t launch_update_b(const JobDesc &J, cudaStream_t st);
