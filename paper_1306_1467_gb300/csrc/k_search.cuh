@@ -224,10 +224,12 @@ struct RunResult {
 // holding chunk u0 + i of the run.  Gives (in every lane) each run's total and
 // its largest / smallest prefix at a valid split, relative to the run start, with
 // the split position (number of entries before it in the whole value order) and
-// the lowest position on ties (INT_MAX if none).
+// the lowest position on ties (INT_MAX if none).  The weights are read with plain
+// loads: the kernels of a round's tail write them later in the same launch, which
+// the read-only path does not allow.
 template <int N>
-__device__ __forceinline__ void rescan_runs(const uint16_t *const (&row)[N], int run, int k, const float *__restrict__ v,
-                                            int lane, RunResult (&res)[N]) {
+__device__ __forceinline__ void rescan_runs(const uint16_t *const (&row)[N], int run, int k, const float *v, int lane,
+                                            RunResult (&res)[N]) {
     DF carry[N], bmax[N], bmn[N];
     int smax[N], smn[N];
     const int nch = run / kChunkElems;
@@ -270,7 +272,7 @@ __device__ __forceinline__ void rescan_runs(const uint16_t *const (&row)[N], int
 #pragma unroll
                 for (int r = 0; r < N; ++r) {
                     const uint32_t e = (j & 1) ? (wd[r][j >> 1] >> 16) : (wd[r][j >> 1] & 0xffffu);
-                    a[r] = df_add_f(a[r], __ldg(v + entry_word(e, j)));
+                    a[r] = df_add_f(a[r], v[entry_word(e, j)]);
                     if (entry_flag(e, j)) {
                         if (df_less(lmx[r], a[r])) { lmx[r] = a[r]; lsx[r] = pos; }
                         if (df_less(a[r], lmn[r])) { lmn[r] = a[r]; lsn[r] = pos; }
@@ -320,8 +322,7 @@ __device__ __forceinline__ void rescan_runs(const uint16_t *const (&row)[N], int
     }
 }
 
-static __device__ RunResult rescan_run(const uint16_t *__restrict__ row, int run, int k, const float *__restrict__ v,
-                                       int lane) {
+static __device__ RunResult rescan_run(const uint16_t *row, int run, int k, const float *v, int lane) {
     const uint16_t *const rows[1] = {row};
     RunResult r[1];
     rescan_runs<1>(rows, run, k, v, lane, r);
