@@ -739,12 +739,20 @@ int vjb_classify(vjb_ctx *c, const uint8_t *pixels, int32_t n, const vjb_stump *
     if (n < 1 || n > (1 << 26)) return fail(VJB_EINVAL, "n = %d outside [1, 2^26]", n);
     if (T < 0) return fail(VJB_EINVAL, "T < 0");
     double half = 0.0;
-    std::vector<ClassStump> cs((size_t)std::max(T, 1));
     for (int t = 0; t < T; ++t) {
         const vjb_stump &s = stumps[t];
         if (s.feature < 0 || s.feature >= c->nfeat || (s.polarity != 1 && s.polarity != -1) || std::isnan(s.alpha))
             return fail(VJB_EINVAL, "stump %d is not a stump of this window size", t);
         half += s.alpha;
+    }
+    std::vector<ClassStump> cs;
+    try {
+        cs.resize((size_t)std::max(T, 1));
+    } catch (const std::bad_alloc &) {
+        return fail(VJB_ENOMEM, "classify: host memory for %d stumps", T);
+    }
+    for (int t = 0; t < T; ++t) {
+        const vjb_stump &s = stumps[t];
         const vjb_feature f = feature_at(c->w, c->h, s.feature);
         cs[(size_t)t] = ClassStump{DevFeature{f.type, f.x, f.y, f.w, f.h, 0, 0, 0}, s.threshold, s.polarity, s.alpha};
     }
