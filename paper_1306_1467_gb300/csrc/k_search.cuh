@@ -417,22 +417,6 @@ __device__ __forceinline__ Candidate load_candidate(const Candidate *p) {
     return c;
 }
 
-// One warp picks job J's stump among its `cnt` re-scanned candidates.
-__device__ __forceinline__ void select_stump_warp(const JobDesc &J, int cnt, int lane) {
-    Candidate b;
-    b.err_hi = INFINITY; b.err_lo = 0.f; b.feature = INT_MAX; b.split = INT_MAX; b.polarity = 1; b.pad = 0;
-    for (int k = lane; k < cnt; k += 32) {
-        const Candidate c = load_candidate(J.cands + k);
-        if (cand_less(c, b)) b = c;
-    }
-#pragma unroll
-    for (int d = 16; d; d >>= 1) {
-        const Candidate o = cand_shfl_xor(b, d);
-        if (cand_less(o, b)) b = o;
-    }
-    if (lane == 0) record_stump(J, cnt, b);
-}
-
 // The whole CTA picks job J's stump among its `cnt` re-scanned candidates.
 static __device__ void select_stump(const JobDesc &J, int cnt) {
     __shared__ Candidate wc[kRescanWarps];

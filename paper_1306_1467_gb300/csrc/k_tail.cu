@@ -301,7 +301,17 @@ __global__ void __launch_bounds__(kTailThreads + 32, 1)
 #pragma unroll
     for (int q = 0; q < kPre; ++q)
         if (first + q * stride < quads) test4(pre[q], first + q * stride);
-    for (int64_t q = first + kPre * stride; q < quads; q += stride) test4(err4[q], q);
+    // the rest of a longer list (windows above 24x24), eight loads in flight a thread:
+    // one after another they took 96 us of the tail at 64x64, 30 more than a grid
+    constexpr int kMore = 8;
+    for (int64_t q0 = first + kPre * stride; q0 < quads; q0 += kMore * stride) {
+        float4 e[kMore];
+#pragma unroll
+        for (int u = 0; u < kMore; ++u) e[u] = err4[min(q0 + u * stride, quads - 1)];
+#pragma unroll
+        for (int u = 0; u < kMore; ++u)
+            if (q0 + u * stride < quads) test4(e[u], q0 + u * stride);
+    }
     if (rank == 0 && tid < (int)(J.nfeat & 3)) test(J.ferr[(J.nfeat & ~(int64_t)3) + tid], (J.nfeat & ~(int64_t)3) + tid);
     cluster.sync();
     const int count = __ldcg(&rs->cand_count);

@@ -109,8 +109,6 @@ struct Candidate {
 constexpr int kLineElems = 64;
 constexpr int kLineBytes = 128;
 constexpr int kBoxLinesMax = 32;
-constexpr int kStageBytes = kBoxLinesMax * kLineBytes;  // 4096
-constexpr int kUnitElems = 512;                         // 32 lanes x 16 entries
 
 // Row layout of the sorted table.  A row holds npad entries (n rounded up to
 // a multiple of 256; entries from n on are padding).  The value order is cut

@@ -100,3 +100,42 @@ def test_a_list_for_the_whole_gpu_costs_little_more():
         return float(np.median(times[3:]))
 
     assert after_search(7, 3, 1) < 4 * after_search(3, 2, 1)
+
+
+@pytest.mark.parametrize("h,w,a", [(25, 28, 1), (32, 32, 2), (40, 37, 3)])
+def test_lists_of_large_windows(h, w, a):
+    """More features than the tail asks for at once (196,608), ties among the last ones."""
+    from paper_1306_1467_gb300 import vjb
+    px, y = _windows(257, h, w, a, 0.2)
+    with vjb.Trainer(0) as tr:
+        tr.prepare(px, y)
+        _, plain = tr.train_strong(2)
+        weights = tr.get_weights()
+        assert tr.round_diag()[0]["candidates"] == _ties(h, w, a)
+    with vjb.Batch(vjb.Batch.table_bytes(257, h, w)) as b:
+        j = b.add_job(px, y, 2)
+        b.train()
+        assert plain == b.stumps(j) and np.array_equal(b.get_weights(j), weights)
+
+
+def test_large_windows_cost_little_more():
+    """What follows the search with one feature listed, 300 samples: 28 us at 24x24
+    and 40 at 48x48 (2,570,880 errors to look through); 65 with a load at a time."""
+    from paper_1306_1467_gb300 import vjb
+
+    def after_search(side):
+        px = np.random.default_rng(side).integers(0, 256, (300, side, side), dtype=np.uint8)
+        with vjb.Trainer(0) as tr:
+            tr.load_windows(px, (np.arange(300) % 3 == 0).astype(np.uint8))
+            tr.build_integral()
+            tr.feature_count()
+            tr.train_strong(3)
+            times = []
+            for _ in range(15):
+                tr.set_timing(True)
+                tr.train_strong(4)
+                t = tr.timing()
+                times.append(t["round_ms_total"] - t["search_ms_total"])
+        return float(np.median(times))
+
+    assert after_search(48) < 1.8 * after_search(24)
