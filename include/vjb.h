@@ -271,6 +271,9 @@ int vjb_get_timing(vjb_ctx *ctx, vjb_timing *out);
  * the result is that of the same sums done one by one on the host; a stump
  * with alpha = +inf (a perfect stump) decides alone.  labels [n] receive
  * C(x), scores [n] (may be NULL) the scores.  Needs vjb_enumerate_haar.
+ * The call's device workspace (pixels, stumps, results) stays with the context
+ * up to 64 MiB, until it is destroyed or loads windows of another shape; a larger
+ * one is freed before the call returns.
  * Errors: VJB_EINVAL (a stump outside the feature list, polarity not +-1,
  * NaN alpha), VJB_ESTATE, VJB_ENOMEM, VJB_ECUDA. */
 int vjb_classify(vjb_ctx *c, const uint8_t *pixels, int32_t n, const vjb_stump *stumps, int32_t T,

@@ -45,8 +45,12 @@ __device__ __forceinline__ void keep_if(uint32_t flag, float before, float g, fl
 // predicated max and min an entry, on the pipe (ALU) that is the busiest after
 // shared memory.  k_screen at 24x24 / 15,000 samples 0.745 -> 0.729 ms, 8,000
 // 0.421 -> 0.411, 4,096 0.223 -> 0.219, 10,963 0.559 -> 0.556, 2,003 0.125 ->
-// 0.1235; 32x32 / 5,003 0.855 -> 0.859.  The kept prefix is added a second
-// time rather than copied: a copy waits for the sum (0.748).
+// 0.1235; 32x32 / 5,003 0.855 -> 0.859.  Of 45 sample counts at 24x24,
+// 29 are faster by 0.4 to 5% and 10 slower: 1,200 and 1,280 by 2 to 3%, 768 by 1
+// to 2%, 2,500, 3,328, 5,000 and 24,000 and their neighbours by 1% or less (the
+// older form in the single pieces that end a row gives 768 back, but takes 2% at
+// 512 and 2,304).  The kept prefix is added a second time rather than copied: a
+// copy waits for the sum (0.748).
 __device__ __forceinline__ void scan_two(uint32_t flag_even, uint32_t flag_odd, float g_even, float g_odd, float &a,
                                          float &even, float &odd, float &mx, float &mn) {
     keep_if(flag_even, a, g_even, even);
@@ -219,114 +223,78 @@ struct RunResult {
     int smx, smn;
 };
 
-// One warp scans lane run k of N rows in double-float, side by side (each is a
-// chain of dependent operations): 32 chunks of 8 entries at a time, lane i
-// holding chunk u0 + i of the run.  Gives (in every lane) each run's total and
-// its largest / smallest prefix at a valid split, relative to the run start, with
-// the split position (number of entries before it in the whole value order) and
-// the lowest position on ties (INT_MAX if none).  The weights are read with plain
-// loads: the kernels of a round's tail write them later in the same launch, which
-// the read-only path does not allow.
-template <int N>
-__device__ __forceinline__ void rescan_runs(const uint16_t *const (&row)[N], int run, int k, const float *v, int lane,
-                                            RunResult (&res)[N]) {
-    DF carry[N], bmax[N], bmn[N];
-    int smax[N], smn[N];
+// One warp scans lane run k of a row in double-float: 32 chunks of 8 entries
+// at a time, lane i holding chunk u0 + i of the run.  Returns (in every lane)
+// the run total and its largest / smallest prefix at a valid split, relative
+// to the run start, with the split position (number of entries before it in
+// the whole value order) and the lowest position on ties (INT_MAX if none).  The
+// weights are read with plain loads: the kernels of a round's tail write them later
+// in the same launch, which the read-only path does not allow.
+static __device__ RunResult rescan_run(const uint16_t *__restrict__ row, int run, int k, const float *v, int lane) {
+    DF carry{0.f, 0.f}, bmax{-INFINITY, 0.f}, bmn{INFINITY, 0.f};
+    int smax = INT_MAX, smn = INT_MAX;
     const int nch = run / kChunkElems;
-    auto load_chunk = [&](int r, int t) {
-        return t < nch ? __ldg(reinterpret_cast<const uint4 *>(row[r] + (size_t)(t * 32 + k) * kChunkElems))
+    auto load_chunk = [&](int t) {
+        return t < nch ? __ldg(reinterpret_cast<const uint4 *>(row + (size_t)(t * 32 + k) * kChunkElems))
                        : make_uint4(0u, 0u, 0u, 0u);
     };
-    uint4 qn[N];  // the next 32 chunks load while these are scanned
-#pragma unroll
-    for (int r = 0; r < N; ++r) {
-        carry[r] = DF{0.f, 0.f};
-        bmax[r] = DF{-INFINITY, 0.f};
-        bmn[r] = DF{INFINITY, 0.f};
-        smax[r] = smn[r] = INT_MAX;
-        qn[r] = load_chunk(r, lane);
-    }
+    uint4 qn = load_chunk(lane);  // the next 32 chunks load while these are scanned
     for (int u0 = 0; u0 < nch; u0 += 32) {
         const int t = u0 + lane;
+        const uint4 q = qn;
+        if (u0 + 32 < nch) qn = load_chunk(t + 32);
+        const uint32_t wd[4] = {q.x, q.y, q.z, q.w};
         const bool have = t < nch;
-        DF a[N], lmx[N], lmn[N];
-        int lsx[N], lsn[N];
-        uint32_t wd[N][4];
-#pragma unroll
-        for (int r = 0; r < N; ++r) {
-            const uint4 q = qn[r];
-            wd[r][0] = q.x; wd[r][1] = q.y; wd[r][2] = q.z; wd[r][3] = q.w;
-            a[r] = DF{0.f, 0.f};
-            lmx[r] = DF{-INFINITY, 0.f};
-            lmn[r] = DF{INFINITY, 0.f};
-            lsx[r] = lsn[r] = INT_MAX;
-        }
-        if (u0 + 32 < nch) {
-#pragma unroll
-            for (int r = 0; r < N; ++r) qn[r] = load_chunk(r, t + 32);
-        }
+        DF a{0.f, 0.f}, lmx{-INFINITY, 0.f}, lmn{INFINITY, 0.f};
+        int lsx = INT_MAX, lsn = INT_MAX;
         if (have) {
 #pragma unroll
             for (int j = 0; j < kChunkElems; ++j) {
-                const int pos = k * run + t * kChunkElems + j + 1;
-#pragma unroll
-                for (int r = 0; r < N; ++r) {
-                    const uint32_t e = (j & 1) ? (wd[r][j >> 1] >> 16) : (wd[r][j >> 1] & 0xffffu);
-                    a[r] = df_add_f(a[r], v[entry_word(e, j)]);
-                    if (entry_flag(e, j)) {
-                        if (df_less(lmx[r], a[r])) { lmx[r] = a[r]; lsx[r] = pos; }
-                        if (df_less(a[r], lmn[r])) { lmn[r] = a[r]; lsn[r] = pos; }
-                    }
+                const uint32_t e = (j & 1) ? (wd[j >> 1] >> 16) : (wd[j >> 1] & 0xffffu);
+                a = df_add_f(a, v[entry_word(e, j)]);
+                if (entry_flag(e, j)) {
+                    const int pos = k * run + t * kChunkElems + j + 1;
+                    if (df_less(lmx, a)) { lmx = a; lsx = pos; }
+                    if (df_less(a, lmn)) { lmn = a; lsn = pos; }
                 }
             }
         }
+        DF x = a;
 #pragma unroll
-        for (int r = 0; r < N; ++r) {
-            DF x = a[r];
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const DF y = df_shfl_up(x, d);
-                if (lane >= d) x = df_add(y, x);
-            }
-            DF excl = df_shfl_up(x, 1);
-            if (lane == 0) excl = DF{0.f, 0.f};
-            const DF tot = df_shfl(x, 31);
-            const DF offs = df_add(carry[r], excl);
-            if (lsx[r] != INT_MAX) {
-                const DF c = df_add(offs, lmx[r]);
-                if (df_less(bmax[r], c)) { bmax[r] = c; smax[r] = lsx[r]; }
-            }
-            if (lsn[r] != INT_MAX) {
-                const DF c = df_add(offs, lmn[r]);
-                if (df_less(c, bmn[r])) { bmn[r] = c; smn[r] = lsn[r]; }
-            }
-            carry[r] = df_add(carry[r], tot);
+        for (int d = 1; d < 32; d <<= 1) {
+            const DF y = df_shfl_up(x, d);
+            if (lane >= d) x = df_add(y, x);
         }
+        DF excl = df_shfl_up(x, 1);
+        if (lane == 0) excl = DF{0.f, 0.f};
+        const DF tot = df_shfl(x, 31);
+        const DF offs = df_add(carry, excl);
+        if (lsx != INT_MAX) {
+            const DF c = df_add(offs, lmx);
+            if (df_less(bmax, c)) { bmax = c; smax = lsx; }
+        }
+        if (lsn != INT_MAX) {
+            const DF c = df_add(offs, lmn);
+            if (df_less(c, bmn)) { bmn = c; smn = lsn; }
+        }
+        carry = df_add(carry, tot);
     }
 #pragma unroll
-    for (int r = 0; r < N; ++r) {
-#pragma unroll
-        for (int d = 16; d; d >>= 1) {
-            const DF om = df_shfl_xor(bmax[r], d);
-            const int os = __shfl_xor_sync(0xffffffffu, smax[r], d);
-            if (df_less(bmax[r], om) || (df_eq(om, bmax[r]) && os < smax[r])) { bmax[r] = om; smax[r] = os; }
-            const DF on = df_shfl_xor(bmn[r], d);
-            const int on_s = __shfl_xor_sync(0xffffffffu, smn[r], d);
-            if (df_less(on, bmn[r]) || (df_eq(on, bmn[r]) && on_s < smn[r])) { bmn[r] = on; smn[r] = on_s; }
-        }
-        res[r].total = carry[r];
-        res[r].mx = bmax[r];
-        res[r].mn = bmn[r];
-        res[r].smx = smax[r];
-        res[r].smn = smn[r];
+    for (int d = 16; d; d >>= 1) {
+        const DF om = df_shfl_xor(bmax, d);
+        const int os = __shfl_xor_sync(0xffffffffu, smax, d);
+        if (df_less(bmax, om) || (df_eq(om, bmax) && os < smax)) { bmax = om; smax = os; }
+        const DF on = df_shfl_xor(bmn, d);
+        const int on_s = __shfl_xor_sync(0xffffffffu, smn, d);
+        if (df_less(on, bmn) || (df_eq(on, bmn) && on_s < smn)) { bmn = on; smn = on_s; }
     }
-}
-
-static __device__ RunResult rescan_run(const uint16_t *row, int run, int k, const float *v, int lane) {
-    const uint16_t *const rows[1] = {row};
-    RunResult r[1];
-    rescan_runs<1>(rows, run, k, v, lane, r);
-    return r[0];
+    RunResult r;
+    r.total = carry;
+    r.mx = bmax;
+    r.mn = bmn;
+    r.smx = smax;
+    r.smn = smn;
+    return r;
 }
 
 // One warp combines a row's 32 lane runs (lane k holds run k's result q):

@@ -9,7 +9,8 @@
 // through shared memory of the cluster.  Rounds of a graph replay, with four
 // kernels (shortlist, re-scan, two updates) before and this now: 31.7 -> 27.6 us
 // at 10x10 / 600, 148.5 -> 145.4 at 24x24 / 2,003, 771.5 -> 769.7 at 24x24 /
-// 15,000 (where four times the SMs shared the FP64 additions before).
+// 15,000 (where four times the SMs shared the FP64 additions before); since, with
+// less code, 27.2, 142.2 and 753.4.
 //
 // Where its 51 k cycles go at 15,000 (clock stamps in a copy): shortlist 5.0,
 // first barrier 1.4, re-scan 9.3, its combination 6.2 with a barrier, update
@@ -77,9 +78,10 @@ __device__ __forceinline__ void sample_barrier() { asm volatile("bar.sync 1, %0;
 // by side for all the blocks).  put(v, block, sum) is called by every lane.
 template <int CTAS, class Put>
 __device__ __forceinline__ void block_sums(const TailShared<CTAS> &S, int rank, int blocks, int warp, int lane, Put put) {
+    constexpr int kWarps = kTailThreads / 32;
 #pragma unroll
-    for (int k = warp; k < 2 * TailShared<CTAS>::kSlots; k += kTailThreads / 32) {
-        const int s = k >> 1, v = k & 1;
+    for (int k0 = 0; k0 < 2 * TailShared<CTAS>::kSlots; k0 += kWarps) {
+        const int s = (k0 + warp) >> 1, v = warp & 1;
         const int blk = s / kTailHalves * (CTAS * kTailHalves) + rank * kTailHalves + s % kTailHalves;
         if (blk >= blocks) continue;
         const float *x = S.samples[s][v];
@@ -99,6 +101,7 @@ __device__ __forceinline__ Candidate no_candidate() {
 // The best of the first `count` places, for every thread.
 __device__ __forceinline__ Candidate best_found(const Candidate *found, int count) {
     Candidate b = no_candidate();
+#pragma unroll 1
     for (int k = 0; k < count; ++k)
         if (cand_less(found[k], b)) b = found[k];
     return b;
@@ -267,15 +270,20 @@ __global__ void __launch_bounds__(kTailThreads + 32, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     RoundState *rs = J.rs;
 
-    // ---- shortlist: everything it reads is asked for at once
+    // ---- shortlist: everything it reads is asked for at once, up to 24 errors a
+    // thread (196,608 features; 24x24 windows have 162,336), then as many again.
+    // The tail with one value after another beyond those, and now: 34 and 27 us at
+    // 32x32, 65 and 35 at 48x48, 145 and 55 at 64x64 (a grid took 30, 45 and 81)
     constexpr int kPre = 6;
     const bool keeper = warp == kTailThreads / 32;
-    const int64_t stride = kTailCtas * kTailThreads, quads = keeper ? 0 : J.nfeat >> 2, first = rank * kTailThreads + tid;
+    const int stride = kTailCtas * kTailThreads, quads = keeper ? 0 : (int)(J.nfeat >> 2), first = rank * kTailThreads + tid;
     const float4 *err4 = reinterpret_cast<const float4 *>(J.ferr);
-    float4 pre[kPre];
+    float4 e[kPre];
+    auto ask = [&](int q0) {
 #pragma unroll
-    for (int q = 0; q < kPre; ++q)
-        if (first + q * stride < quads) pre[q] = err4[first + q * stride];
+        for (int u = 0; u < kPre; ++u) e[u] = err4[min(q0 + u * stride, quads - 1)];
+    };
+    if (first < quads) ask(first);
     float m = INFINITY;
     for (int i = tid; i < nbmin; i += (int)blockDim.x) m = fminf(m, bmin[i]);
     const int32_t status = rs->status, forced = rs->forced, r0 = rs->rounds;
@@ -290,27 +298,26 @@ __global__ void __launch_bounds__(kTailThreads + 32, 1)
     auto test = [&](float e, int64_t f) {
         if (e <= thr) J.cand_ids[atomicAdd(&rs->cand_count, 1)] = (int32_t)f;  // (the count is zero between rounds)
     };
-    auto test4 = [&](const float4 &e, int64_t q) {
-        if (fminf(fminf(e.x, e.y), fminf(e.z, e.w)) <= thr) {
-            test(e.x, 4 * q);
-            test(e.y, 4 * q + 1);
-            test(e.z, 4 * q + 2);
-            test(e.w, 4 * q + 3);
+    // few threads list anything: those read their four errors again, so that one
+    // piece of code serves all of them (after a long search the tail's code is
+    // fetched anew, and its length counts: rounds at 24x24 / 2,003 146.6 us with a
+    // test for each of 14 loads and a second form of the re-scan, 142.2 now)
+    for (int q0 = first; q0 < quads;) {
+        uint32_t hits = 0u;
+#pragma unroll
+        for (int u = 0; u < kPre; ++u)
+            if (q0 + u * stride < quads && fminf(fminf(e[u].x, e[u].y), fminf(e[u].z, e[u].w)) <= thr) hits |= 1u << u;
+        while (hits) {
+            const int q = q0 + (__ffs(hits) - 1) * stride;
+            hits &= hits - 1u;
+            const float4 x = err4[q];
+            test(x.x, 4 * (int64_t)q);
+            test(x.y, 4 * (int64_t)q + 1);
+            test(x.z, 4 * (int64_t)q + 2);
+            test(x.w, 4 * (int64_t)q + 3);
         }
-    };
-#pragma unroll
-    for (int q = 0; q < kPre; ++q)
-        if (first + q * stride < quads) test4(pre[q], first + q * stride);
-    // the rest of a longer list (windows above 24x24), eight loads in flight a thread:
-    // one after another they took 96 us of the tail at 64x64, 30 more than a grid
-    constexpr int kMore = 8;
-    for (int64_t q0 = first + kPre * stride; q0 < quads; q0 += kMore * stride) {
-        float4 e[kMore];
-#pragma unroll
-        for (int u = 0; u < kMore; ++u) e[u] = err4[min(q0 + u * stride, quads - 1)];
-#pragma unroll
-        for (int u = 0; u < kMore; ++u)
-            if (q0 + u * stride < quads) test4(e[u], q0 + u * stride);
+        q0 += kPre * stride;
+        if (q0 < quads) ask(q0);
     }
     if (rank == 0 && tid < (int)(J.nfeat & 3)) test(J.ferr[(J.nfeat & ~(int64_t)3) + tid], (J.nfeat & ~(int64_t)3) + tid);
     cluster.sync();
@@ -326,32 +333,17 @@ __global__ void __launch_bounds__(kTailThreads + 32, 1)
         return;  // the whole cluster
     }
 
-    // ---- compensated re-scan: a warp per run, a feature's 32 runs on 16 SMs; with
-    // more than 8 features two runs a warp, the same one of two features 8 apart
-    // (side by side; one after the other and one warp combining every feature, 15
-    // features took 55 us after the search at 15,000 samples and 49 at 600; now 35
-    // and 28)
-    constexpr int kWarps = kTailCtas * (kTailThreads / 32);
-    static_assert(kTailCands * 32 <= 2 * kWarps && kWarps % 32 == 0, "at most two runs a warp");
-    const int i = rank + kTailCtas * warp, i2 = i + kWarps;
-    if (!keeper && i < count * 32) {
-        auto row = [&](int at) { return J.rows + (size_t)__ldcg(J.cand_ids + (at >> 5)) * J.npad; };
-        auto push = [&](int at, const RunResult &r) {
-            if (lane < kTailCtas) cluster.map_shared_rank(&S, lane)->runs[at] = r;  // to every CTA
-        };
-        if (i2 < count * 32) {
-            const uint16_t *const rows[2] = {row(i), row(i2)};
-            RunResult r[2];
-            rescan_runs<2>(rows, J.npad / 32, i & 31, J.v, lane, r);
-            push(i, r[0]);
-            push(i2, r[1]);
-        } else {
-            push(i, rescan_run(row(i), J.npad / 32, i & 31, J.v, lane));
-        }
+    // ---- compensated re-scan: a warp per run, a feature's 32 runs on 16 SMs (two
+    // runs side by side for lists above 8 gained nothing)
+    for (int i = rank + kTailCtas * warp; !keeper && i < count * 32; i += kTailCtas * (kTailThreads / 32)) {
+        const int32_t f = __ldcg(J.cand_ids + (i >> 5));
+        const RunResult r = rescan_run(J.rows + (size_t)f * J.npad, J.npad / 32, i & 31, J.v, lane);
+        if (lane < kTailCtas) cluster.map_shared_rank(&S, lane)->runs[i] = r;  // to every CTA
     }
     cluster.sync();
     // the stump, found by every CTA for itself: a warp per feature, then a look at
-    // each
+    // each (15 features at 15,000 samples and at 600 take 35 and 28 us after the
+    // search; 55 and 49 when one warp combined them all)
     if (warp < count) {
         const Candidate cd = combine_runs(J, __ldcg(J.cand_ids + warp), S.runs[warp * 32 + lane], lane);
         if (lane == 0) S.found[warp] = cd;
@@ -370,8 +362,8 @@ __global__ void __launch_bounds__(kTailThreads + 32, 1)
 // What follows the search (events), by features listed; in brackets with one CTA
 // of the last feature doing the update, 256 samples after another:
 //   15,000 samples       21: 43 us (178)   300: 51 (182)   5,050: 248 (412)
-//   32,766 samples       21: 57 us (403)   300: 82 (414)   5,050: 628 (800)
-//   600 samples          21: 29 us (35)    595: 43 (41)    5,050: 147 (153)
+//   32,766 samples       21: 57 us (403)   300: 82 (414)   5,050: 602 (800)
+//   600 samples          21: 29 us (35)    595: 42 (40)    5,050: 146 (153)
 //   20x20 / 19,997       78,460: 5.3 ms (6.0), the whole round
 __global__ void __launch_bounds__(kTailThreads + 32, 2) k_plateau(const __grid_constant__ JobDesc J) {
     RoundState *rs = J.rs;

@@ -761,10 +761,11 @@ int vjb_classify(vjb_ctx *c, const uint8_t *pixels, int32_t n, const vjb_stump *
     if (rc) return rc;
     // Windows go to the device a part at a time, in two buffers, so that a part
     // is classified while the next is copied (86 MB of 24x24 windows: the copy
-    // alone takes 490 us, the kernels 302; the call 831 us with parts of 24 MiB,
-    // 886 with 8 and 1,017 with 4, and 1,814 with one copy, integral images in
-    // memory and buffers allocated and freed).  Windows too large for shared
-    // memory go through integral images in memory, whole.
+    // alone takes 490 us, the kernels 302, the call about 725.  Parts of 24 MiB
+    // against 8 and 4, when the call took 100 us more: 831, 886 and 1,017; with one
+    // copy, integral images in memory and buffers allocated and freed 1,814).
+    // Windows too large for shared memory go through integral images in memory,
+    // whole.
     const size_t hw = (size_t)c->h * c->w;
     const bool fused = classify_fits(c->h, c->w);
     const int part = fused ? (int)std::min<size_t>((size_t)(n + 31) / 32 * 32, std::max<size_t>(32, (kClassifyPartBytes / hw) / 32 * 32)) : n;

@@ -1,5 +1,5 @@
-"""Rounds by the length of their list: of one feature a warp, of two runs a warp
-(above 8), the longest that the cluster keeps (16), the shortest that goes to the
+"""Rounds by the length of their list: of a run a warp, of two runs a warp (above
+8), the longest that the cluster keeps (16), the shortest that goes to the
 whole GPU (17), one with a feature for every block, and several for each.
 
 Windows of grey columns, with faces and non-faces told apart (but for a share of
@@ -119,8 +119,8 @@ def test_lists_of_large_windows(h, w, a):
 
 
 def test_large_windows_cost_little_more():
-    """What follows the search with one feature listed, 300 samples: 28 us at 24x24
-    and 40 at 48x48 (2,570,880 errors to look through); 65 with a load at a time."""
+    """What follows the search with one feature listed, 300 samples: 25 us at 24x24
+    and 35 at 48x48 (2,570,880 errors to look through); 65 with a load at a time."""
     from paper_1306_1467_gb300 import vjb
 
     def after_search(side):
