@@ -9,8 +9,8 @@
 // through shared memory of the cluster.  Rounds of a graph replay, with four
 // kernels (shortlist, re-scan, two updates) before and this now: 31.7 -> 27.6 us
 // at 10x10 / 600, 148.5 -> 145.4 at 24x24 / 2,003, 771.5 -> 769.7 at 24x24 /
-// 15,000 (where four times the SMs shared the FP64 additions before); since, with
-// less code, 27.2, 142.2 and 753.4.
+// 15,000 (where four times the SMs shared the FP64 additions before); by now, with
+// less code here and a faster search, 27.2, 142.2 and 753.4.
 //
 // Where its 51 k cycles go at 15,000 (clock stamps in a copy): shortlist 5.0,
 // first barrier 1.4, re-scan 9.3, its combination 6.2 with a barrier, update
