@@ -48,3 +48,41 @@ def test_window_sizes_side_by_side():
                 raise got
             assert np.array_equal(got, alone[s]), s
         assert len(together[s]) == 400
+
+
+def test_training_side_by_side():
+    """Rounds whose lists go to the whole GPU (equal rows: every column pair of one
+    height ties with the others), of four contexts at once."""
+    from paper_1306_1467_gb300 import vjb
+
+    def run(k, out):
+        rng = np.random.default_rng(k)
+        n, h = 3000 + 1111 * k, 8 + 6 * k
+        y = (np.arange(n) % 3 == 0).astype(np.uint8)
+        px = np.repeat((rng.integers(0, 200, (n, 1, 2)) + 20 * y[:, None, None] * np.array([0, 1])).astype(np.uint8), h, axis=1)
+        try:
+            with vjb.Trainer(0) as tr:
+                tr.prepare(px, y)
+                for _ in range(10):
+                    tr.load_windows(px, y)
+                    tr.build_integral()
+                    tr.feature_count()
+                    out.append((tr.train_strong(20), tr.get_weights().tobytes(), max(d["candidates"] for d in tr.round_diag())))
+        except Exception as e:  # for the thread that compares
+            out.append(e)
+
+    alone, together = [], [[] for _ in range(4)]
+    for k in range(4):
+        out = []
+        run(k, out)
+        if isinstance(out[-1], Exception):
+            raise out[-1]
+        alone.append(out[0])
+        assert out[0][2] > 16
+    threads = [threading.Thread(target=run, args=(k, together[k])) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for k in range(4):
+        assert together[k] == [alone[k]] * 10
