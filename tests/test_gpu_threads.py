@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 SIZES = [(6, 6), (10, 10), (24, 24), (32, 32)]
 
 
-def _work(h, w, times, out):
+def _steps(h, w, times, out):
     from paper_1306_1467_gb300 import vjb
     rng = np.random.default_rng(h * 100 + w)
     px = rng.integers(0, 256, (64, h, w), dtype=np.uint8)
@@ -35,9 +35,9 @@ def test_window_sizes_side_by_side():
     alone, together = {}, {s: [] for s in SIZES}
     for s in SIZES:
         out = []
-        _work(*s, 1, out)
+        _steps(*s, 1, out)
         alone[s] = out[0]
-    threads = [threading.Thread(target=_work, args=(*s, 400, together[s])) for s in SIZES]
+    threads = [threading.Thread(target=_steps, args=(*s, 400, together[s])) for s in SIZES]
     for t in threads:
         t.start()
     for t in threads:
